@@ -915,12 +915,6 @@ gbsp_status jds_build_impl(const Mat &A, const gbsp_jds_opts &o, const gbsp_jds_
 
 // ------------------------------------------------------------ transpose --
 
-__global__ void row_of_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr, int32_t *row_of) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rows) return;
-    for (int32_t k = row_ptr[r]; k < row_ptr[r + 1]; ++k) row_of[k] = (int32_t)r;
-}
-
 __global__ void col_count_kernel(int64_t nnz, const int32_t *__restrict__ col, int32_t *count) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < nnz) atomicAdd(count + col[k], 1);
@@ -1030,8 +1024,26 @@ gbsp_status jds_values_launch(const Mat &J, const void *src, cudaStream_t s) {
 }
 
 gbsp_status transpose_workspace_impl(const Mat &A, int64_t *bytes) {
-    *bytes = align256(4 * A.nnz) * 2 + sort_ws_bytes(A.nnz) + align256(scan_ws_bytes(A.n_cols + 1)) + 256;
+    *bytes = transpose_split_fits(A)
+                 ? transpose_split_bytes(A)
+                 : align256(4 * A.nnz) * 2 + sort_ws_bytes(A.nnz) + align256(scan_ws_bytes(A.n_cols + 1)) + 256;
     return GBSP_OK;
+}
+
+static void transpose_handle(const Mat &A, const gbsp_transpose_buffers &b, Mat *T) {
+    T->kind = KIND_CRS;
+    T->n_rows = A.n_cols;
+    T->n_cols = A.n_rows;
+    T->nnz = A.nnz;
+    T->dtype = A.dtype;
+    T->device = A.device;
+    T->row_ptr = b.t_row_ptr;
+    T->col = b.t_col;
+    T->val = b.t_val;
+    T->tmap = b.tmap;
+    T->transpose_src = &A;
+    crs_default_opts(*T);
+    T->kopt.accum = A.kopt.accum;
 }
 
 gbsp_status transpose_build_impl(const Mat &A, const gbsp_transpose_buffers &b, int64_t ws_bytes,
@@ -1042,6 +1054,12 @@ gbsp_status transpose_build_impl(const Mat &A, const gbsp_transpose_buffers &b, 
         set_error("transpose workspace too small: %lld < %lld", (long long)ws_bytes, (long long)need);
         return GBSP_ERR_NOMEM;
     }
+    if (transpose_split_fits(A)) {
+        transpose_handle(A, b, T);
+        return transpose_split_build(A, b, s);
+    }
+    // more columns than the split's buckets hold: byte-wise radix sort of
+    // (column, entry), then rows and values gathered by entry
     char *p = static_cast<char *>(b.workspace);
     int32_t *row_of = reinterpret_cast<int32_t *>(p);
     p += align256(4 * A.nnz);
@@ -1053,7 +1071,7 @@ gbsp_status transpose_build_impl(const Mat &A, const gbsp_transpose_buffers &b, 
     GBSP_CUDA(cudaMemsetAsync(b.t_row_ptr, 0, 4 * (A.n_cols + 1), s));
     if (A.nnz > 0) {
         const unsigned gk = (unsigned)ceil_div(A.nnz, 256);
-        row_of_kernel<<<(unsigned)ceil_div(A.n_rows, 256), 256, 0, s>>>(A.n_rows, A.row_ptr, row_of);
+        row_of_launch(A, row_of, s);
         col_count_kernel<<<gk, 256, 0, s>>>(A.nnz, A.col, b.t_row_ptr);
         copy_keys_kernel<<<gk, 256, 0, s>>>(A.nnz, A.col, keys);
         GBSP_LAUNCH_CHECK("transpose counts");
@@ -1068,19 +1086,7 @@ gbsp_status transpose_build_impl(const Mat &A, const gbsp_transpose_buffers &b, 
     gbsp_status st = scan_exclusive(b.t_row_ptr, A.n_cols, b.t_row_ptr, b.t_row_ptr + A.n_cols, scan_ws, s);
     if (st != GBSP_OK) return st;
 
-    T->kind = KIND_CRS;
-    T->n_rows = A.n_cols;
-    T->n_cols = A.n_rows;
-    T->nnz = A.nnz;
-    T->dtype = A.dtype;
-    T->device = A.device;
-    T->row_ptr = b.t_row_ptr;
-    T->col = b.t_col;
-    T->val = b.t_val;
-    T->tmap = b.tmap;
-    T->transpose_src = &A;
-    crs_default_opts(*T);
-    T->kopt.accum = A.kopt.accum;
+    transpose_handle(A, b, T);
     return transpose_values_impl(*T, s);
 }
 

@@ -173,6 +173,12 @@ gbsp_status jds_values_launch(const Mat &J, const void *src, cudaStream_t s);
 gbsp_status gather_values_launch(int64_t n, const int32_t *map, const void *src, void *dst, int dtype,
                                  cudaStream_t s);
 
+// transpose.cu ----------------------------------------------------------
+bool transpose_split_fits(const Mat &A);
+int64_t transpose_split_bytes(const Mat &A);
+gbsp_status transpose_split_build(const Mat &A, const gbsp_transpose_buffers &b, cudaStream_t s);
+void row_of_launch(const Mat &A, int32_t *row_of, cudaStream_t s);  // row of every entry
+
 }  // namespace gbsp
 
 struct gbsp_mat : gbsp::Mat {};
