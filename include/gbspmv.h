@@ -113,7 +113,9 @@ typedef enum { GBSP_BASIS_PERMUTED = 0, GBSP_BASIS_ORIGINAL = 1 } gbsp_basis;
 typedef enum { GBSP_ACC_PLAIN = 0, GBSP_ACC_COMPENSATED = 1 } gbsp_accum;
 
 /* CRS kernel choice.  VECTOR: `lanes` threads of a warp per row, each warp
- * working on `rows_per_warp` rows at a time (lanes * rows in flight).
+ * working on `rows_per_warp` rows at a time (lanes * rows in flight); rows
+ * of more than 16 * lanes entries are summed by the whole warp, and with one
+ * lane a row those of 9 to 128 entries by eight lanes.
  * TILED: rows grouped into tiles of `tile` merge items (rows + entries);
  * a persistent CTA streams its tiles' val, col and row_ptr slices into
  * shared memory with bulk asynchronous copies (a producer warp, mbarrier

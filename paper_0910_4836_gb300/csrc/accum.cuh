@@ -77,7 +77,7 @@ template <> struct Acc<VM_F32C> {
     __device__ __forceinline__ void merge(const Acc &o) {
         float t;
         two_sum(s, o.s, s, t);
-        c += o.c + t;
+        c = (c + o.c) + t;  // symmetric, so both lanes of a pair get the same bits
     }
     __device__ __forceinline__ void shfl_xor_merge(int off) {
         Acc o;

@@ -15,6 +15,7 @@
 
 #include "accum.cuh"
 #include "internal.cuh"
+#include "rows.cuh"
 #include "sm100.cuh"
 
 namespace gbsp {
@@ -53,6 +54,11 @@ __device__ void batch_crs_rows(const BatchMat &m, int64_t rb, int64_t re) {
     const T *val = static_cast<const T *>(m.val);
     const T *x = static_cast<const T *>(m.x);
     T *y = static_cast<T *>(m.y);
+    if (L == 1) {
+        for (int64_t base = rb + (int64_t)wid * 32; base < re; base += kBatchThreads)
+            crs_short_rows<VM, 1>(base, re, m.row_ptr, m.col, val, x, m.ldx, y, m.ldy, 0);
+        return;
+    }
     for (int64_t base = rb + (int64_t)wid * G; base < re; base += (int64_t)(kBatchThreads / 32) * G) {
         const int64_t r = base + grp;
         int k0 = 0, k1 = 0;
@@ -60,11 +66,15 @@ __device__ void batch_crs_rows(const BatchMat &m, int64_t rb, int64_t re) {
             k0 = __ldg(m.row_ptr + r);
             k1 = __ldg(m.row_ptr + r + 1);
         }
+        const unsigned lmask = k1 - k0 > vector_long_row<L>() ? 1u : 0u;
+        if (lmask) k1 = k0;
         Acc<VM> acc;
         acc.init();
         for (int j = k0 + gl; j < k1; j += L) acc.add(__ldg(val + j), ld_vec(x + (int64_t)__ldg(m.col + j) * m.ldx));
         group_reduce<L, VM>(acc);
-        if (gl == 0 && r < re) y[r * m.ldy] = acc.result();
+        if (gl == 0 && r < re && !lmask) y[r * m.ldy] = acc.result();
+        if (__any_sync(0xffffffffu, lmask != 0))
+            crs_warp_long_rows<VM>(gl == 0, lmask, r, 1, m.row_ptr, m.col, val, x, m.ldx, y, m.ldy, 0);
     }
 }
 

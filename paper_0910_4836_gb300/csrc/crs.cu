@@ -9,9 +9,10 @@
 // butterfly of warp shuffles; when a group holds as many rows as it has
 // lanes, by a reduce-scatter that leaves each lane one row's total (same
 // tree, fewer FP64 additions: on GB300 each one is a full-rate-limited FP64
-// instruction).  In a warp whose rows include one longer than kLongRow, the
-// groups take their rows one at a time and the long rows are then summed by
-// the whole warp.
+// instruction).  Rows of more than 16 L entries are cut out of their group's
+// loop and summed by the whole warp afterwards.  With one lane a row
+// (crs_short_rows) rows are sorted into three classes by length: one lane,
+// eight lanes, the whole warp.
 //
 // RUNS: as VECTOR, but a group's rows are consecutive and its lanes stride
 // through their entries as one run (below).
@@ -31,112 +32,113 @@
 namespace gbsp {
 
 constexpr int kThreads = 256;
-// Row length beyond which a row is summed by the whole warp instead of its
-// lane group: VECTOR (lanes run to the group's longest row) and RUNS (whose
-// groups share one run, so a long row would hold its whole group).
-constexpr int kLongRow = 512;
+// RUNS: row length beyond which a row is summed by the whole warp (a group's
+// rows share one run, so a long row would hold its whole group).
 constexpr int kRunsLongRow = 64;
 
-// Flagged rows with the whole warp on each row in turn.  Every lane passes
-// its group's mask (bit i: row first + i * step is long; only `leader`
-// lanes' masks are read); lanes stride through a row four loads deep, then
-// a full-warp sum.  Called only from the out-of-line long-row steps below,
-// so it does not weigh on the common path's registers.
-template <int VM>
-__device__ __forceinline__ void crs_warp_long_rows(bool leader, unsigned mask, int64_t first, int64_t step,
-                                                const int32_t *__restrict__ row_ptr,
-                                                const int32_t *__restrict__ col,
-                                                const typename ValT<VM>::T *__restrict__ val,
-                                                const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
-                                                typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
-    typedef typename ValT<VM>::T T;
-    const int lane = threadIdx.x & 31;
-    unsigned todo = __ballot_sync(0xffffffffu, leader && mask != 0);
-    while (todo) {
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        unsigned m = __shfl_sync(0xffffffffu, mask, src);
-        const int64_t f = __shfl_sync(0xffffffffu, first, src);
-        while (m) {
-            const int64_t r = f + (int64_t)(__ffs(m) - 1) * step;
-            m &= m - 1;
-            const int s0 = __ldg(row_ptr + r), s1 = __ldg(row_ptr + r + 1);
-            Acc<VM> a;
-            a.init();
-            for (int j = s0 + lane; j < s1; j += 4 * 32) {
-                int c[4];
-                T v[4];
+// The group's R partial sums over its L lanes (R, L powers of two) and the
+// stores: a reduce-scatter, in which each lane trades half of its sums with
+// its partner as long as it holds several, then adds its partner's.  Lane gl
+// ends with row i = gl / (L / R) (R < L) or rows (R / L) gl + q, after
+// R - 1 or L - 1 (+ log2(L / R)) additions instead of R log2(L); on GB300
+// each one is a full FP64 instruction.  The tree per row is the xor butterfly
+// of group_reduce with some additions' operands swapped, which the merges do
+// not notice: every row's sum is bit-identical to it.  Rows of the group are
+// first + i step; those flagged in lmask are not stored.
+template <int VM, int L, int R>
+__device__ __forceinline__ void scatter_store(Acc<VM> (&acc)[R], int64_t first, int64_t step, unsigned lmask,
+                                              int64_t n_rows, typename ValT<VM>::T *__restrict__ y, int64_t ldy,
+                                              int accumulate) {
+    const int gl = (threadIdx.x & 31) % L;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool ok = j + 32 * u < s1;
-                    c[u] = ok ? __ldg(col + j + 32 * u) : -1;
-                    v[u] = ok ? __ldg(val + j + 32 * u) : T(0);
-                }
+    for (int o = L / 2, h = R / 2; o > 0; o >>= 1, h >>= 1) {
+        if (h > 0) {
+            const bool up = (gl & o) != 0;
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (c[u] >= 0) a.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
+            for (int k = 0; k < h; ++k) {
+                Acc<VM> send = up ? acc[k] : acc[k + h];
+                Acc<VM> keep = up ? acc[k + h] : acc[k];
+                keep.merge_shfl_xor(send, o);
+                acc[k] = keep;
             }
-            group_reduce<32, VM>(a);
-            if (lane == 0) {
-                if (accumulate) a.add_value(y[r * ldy]);
-                y[r * ldy] = a.result();
-            }
+        } else {
+            acc[0].shfl_xor_merge(o);
+        }
+    }
+    constexpr int Q = R > L ? R / L : 1, P = L > R ? L / R : 1;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int i = Q * (gl / P) + q;
+        const int64_t r = first + i * step;
+        if (gl % P == 0 && r < n_rows && !((lmask >> i) & 1u)) {
+            if (accumulate) acc[q].add_value(y[r * ldy]);
+            y[r * ldy] = acc[q].result();
         }
     }
 }
 
-// The step of a warp that holds a very long row (heavy-tailed row lengths),
-// for VECTOR and RUNS alike: group g's rows are first_g + i step, i < R.
-// Rows up to `thr` entries are summed one at a time by their group's L lanes
-// (four loads in flight per lane, then the group's butterfly); longer rows,
-// which would keep their group busy long after the rest of the warp is done,
-// are then summed by the whole warp.  Out of line, and light on registers,
-// so that the common step keeps its own.
-template <int VM, int L>
-__device__ __noinline__ void crs_step_with_long_rows(int R, int64_t first, int64_t step, int thr, int64_t n_rows,
-                                                     const int32_t *__restrict__ row_ptr,
-                                                     const int32_t *__restrict__ col,
-                                                     const typename ValT<VM>::T *__restrict__ val,
-                                                     const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
-                                                     typename ValT<VM>::T *__restrict__ y, int64_t ldy,
-                                                     int accumulate) {
+// One VECTOR step (group rows first + i G, i < R): the loop over the entries,
+// `len` the group's longest row.
+template <int VM, int L, int R>
+__device__ __forceinline__ void vector_sums(Acc<VM> (&acc)[R], const int (&k0)[R], const int (&k1)[R], int len,
+                                            const int32_t *__restrict__ col,
+                                            const typename ValT<VM>::T *__restrict__ val,
+                                            const typename ValT<VM>::T *__restrict__ x, int64_t ldx) {
     typedef typename ValT<VM>::T T;
-    const int gl = (threadIdx.x & 31) % L;
-    unsigned lmask = 0;
-#pragma unroll 1
-    for (int i = 0; i < R; ++i) {
-        const int64_t r = first + i * step;
-        int s0 = 0, s1 = 0;
-        if (r < n_rows) {
-            s0 = __ldg(row_ptr + r);
-            s1 = __ldg(row_ptr + r + 1);
-        }
-        if (s1 - s0 > thr) {
-            lmask |= 1u << i;
-            s1 = s0;
-        }
-        Acc<VM> a;
-        a.init();
-        for (int j = s0 + gl; j < s1; j += 4 * L) {
-            int c[4];
-            T v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool ok = j + L * u < s1;
-                c[u] = ok ? __ldg(col + j + L * u) : -1;
-                v[u] = ok ? __ldg(val + j + L * u) : T(0);
-            }
+    for (int i = 0; i < R; ++i) acc[i].init();
+    for (int j = (threadIdx.x & 31) % L; j < len; j += L) {
+        int c[R];
+        T v[R];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c[u] >= 0) a.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
+        for (int i = 0; i < R; ++i) {
+            const int k = k0[i] + j;
+            const bool ok = k < k1[i];
+            // read-only path, not evict-first: a lane group touches a
+            // sector in several iterations, so it must survive in L1/L2
+            c[i] = ok ? __ldg(col + k) : -1;
+            v[i] = ok ? __ldg(val + k) : T(0);
         }
-        group_reduce<L, VM>(a);
-        if (gl == 0 && r < n_rows && !((lmask >> i) & 1u)) {
-            if (accumulate) a.add_value(y[r * ldy]);
-            y[r * ldy] = a.result();
-        }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+            if (c[i] >= 0) acc[i].add(v[i], ld_vec(x + (int64_t)c[i] * ldx));
     }
-    crs_warp_long_rows<VM>(gl == 0, lmask, first, step, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+}
+
+// A VECTOR step whose warp holds a row longer than vector_long_row: such
+// rows are left out of the groups' loops and summed afterwards by the whole
+// warp.  Out of line, so that the common step keeps its registers and code
+// (with the cut in the common step the 4 x 4 shape took 76 us instead of 65 us
+// on the HH-like matrix of N = 1,201,200).
+template <int VM, int L, int R>
+__device__ __noinline__ void vector_step_cut(int64_t first, int64_t n_rows, const int32_t *__restrict__ row_ptr,
+                                             const int32_t *__restrict__ col,
+                                             const typename ValT<VM>::T *__restrict__ val,
+                                             const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                                             typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    constexpr int G = 32 / L;
+    int k0[R], k1[R];
+    int len = 0;
+    unsigned lmask = 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int64_t r = first + i * G;
+        k0[i] = 0;
+        k1[i] = 0;
+        if (r < n_rows) {
+            k0[i] = __ldg(row_ptr + r);
+            k1[i] = __ldg(row_ptr + r + 1);
+        }
+        if (k1[i] - k0[i] > vector_long_row<L>()) {
+            lmask |= 1u << i;
+            k1[i] = k0[i];
+        }
+        len = max(len, k1[i] - k0[i]);
+    }
+    Acc<VM> acc[R];
+    vector_sums<VM, L, R>(acc, k0, k1, len, col, val, x, ldx);
+    scatter_store<VM, L, R>(acc, first, G, lmask, n_rows, y, ldy, accumulate);
+    crs_warp_long_rows<VM>((threadIdx.x & 31) % L == 0, lmask, first, G, row_ptr, col, val, x, ldx, y, ldy, accumulate);
 }
 
 // The occupancy hint (stated for 256-thread CTAs; the kernel is launched in
@@ -149,11 +151,9 @@ crs_vector_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                   const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                   const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
                   typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
-    typedef typename ValT<VM>::T T;
     constexpr int G = 32 / L;
     constexpr int RW = G * R;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / L, gl = lane % L;
+    const int grp = (threadIdx.x & 31) / L;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t base = warp * RW; base < n_rows; base += nwarp * RW) {
@@ -170,69 +170,27 @@ crs_vector_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
             }
             len = max(len, k1[i] - k0[i]);
         }
-        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)kLongRow) {
-            crs_step_with_long_rows<VM, L>(R, base + grp, G, kLongRow, n_rows, row_ptr, col, val, x, ldx, y, ldy,
-                                              accumulate);
+        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)vector_long_row<L>()) {
+            vector_step_cut<VM, L, R>(base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
             continue;
         }
         Acc<VM> acc[R];
-#pragma unroll
-        for (int i = 0; i < R; ++i) acc[i].init();
-        for (int j = gl; j < len; j += L) {
-            int c[R];
-            T v[R];
-#pragma unroll
-            for (int i = 0; i < R; ++i) {
-                const int k = k0[i] + j;
-                const bool ok = k < k1[i];
-                // read-only path, not evict-first: a lane group touches a
-                // sector in several iterations, so it must survive in L1/L2
-                c[i] = ok ? __ldg(col + k) : -1;
-                v[i] = ok ? __ldg(val + k) : T(0);
-            }
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-                if (c[i] >= 0) acc[i].add(v[i], ld_vec(x + (int64_t)c[i] * ldx));
-        }
-        if (R == L && VM != VM_F32C) {
-            // reduce-scatter: log2(L) steps, each lane trading half of its
-            // partial sums with its partner, so lane gl ends with row gl's
-            // total after L - 1 additions instead of R log2(L).  The tree per
-            // row is the xor butterfly of group_reduce with some additions'
-            // operands swapped, which plain sums do not notice: every row's
-            // sum is bit-identical to it.  (The compensated merge is not
-            // symmetric in its error terms, so FP32C keeps the butterfly.)
-#pragma unroll
-            for (int o = L / 2, h = R / 2; o > 0; o >>= 1, h >>= 1) {
-                const bool up = (gl & o) != 0;
-#pragma unroll
-                for (int k = 0; k < h; ++k) {
-                    Acc<VM> send = up ? acc[k] : acc[k + h];
-                    Acc<VM> keep = up ? acc[k + h] : acc[k];
-                    keep.merge_shfl_xor(send, o);
-                    acc[k] = keep;
-                }
-            }
-            const int64_t r = base + gl * G + grp;
-            if (r < n_rows) {
-                if (accumulate) acc[0].add_value(y[r * ldy]);
-                y[r * ldy] = acc[0].result();
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < R; ++i) group_reduce<L, VM>(acc[i]);
-            if (gl == 0) {
-#pragma unroll
-                for (int i = 0; i < R; ++i) {
-                    const int64_t r = base + i * G + grp;
-                    if (r < n_rows) {
-                        if (accumulate) acc[i].add_value(y[r * ldy]);
-                        y[r * ldy] = acc[i].result();
-                    }
-                }
-            }
-        }
+        vector_sums<VM, L, R>(acc, k0, k1, len, col, val, x, ldx);
+        scatter_store<VM, L, R>(acc, base + grp, G, 0u, n_rows, y, ldy, accumulate);
     }
+}
+
+// VECTOR with one lane a row (short rows).
+template <int VM, int R>
+__global__ void __launch_bounds__(kThreads, R == 1 ? 6 : 5)
+crs_short_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
+                 const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
+                 const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                 typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t base = warp * 32 * R; base < n_rows; base += nwarp * 32 * R)
+        crs_short_rows<VM, R>(base, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
 }
 
 // Park a lane's running sum in its row's slot.  Indices are compile-time
@@ -257,34 +215,6 @@ __device__ __forceinline__ void park(Acc<VM> (&part)[R], int cur, const Acc<VM> 
 // entries per lane are loaded and gathered before any product is formed (U
 // gathers in flight).
 constexpr int kRunsU = 4;
-
-// Reduce-scatter of the R row slots over the group's L lanes, then the
-// stores (rows flagged in lmask are not stored).
-template <int VM, int L, int R>
-__device__ __forceinline__ void runs_store(Acc<VM> (&part)[R], int64_t rg, unsigned lmask, int64_t n_rows,
-                                           typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
-    const int gl = (threadIdx.x & 31) % L;
-#pragma unroll
-    for (int o = L / 2, h = R / 2; o > 0; o >>= 1, h >>= 1) {
-        const bool up = (gl & o) != 0;
-#pragma unroll
-        for (int k = 0; k < h; ++k) {
-            Acc<VM> send = up ? part[k] : part[k + h];
-            Acc<VM> keep = up ? part[k + h] : part[k];
-            keep.merge_shfl_xor(send, o);
-            part[k] = keep;
-        }
-    }
-    constexpr int Q = R / L;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int64_t r = rg + (int64_t)Q * gl + q;
-        if (r < n_rows && !((lmask >> (Q * gl + q)) & 1u)) {
-            if (accumulate) part[q].add_value(y[r * ldy]);
-            y[r * ldy] = part[q].result();
-        }
-    }
-}
 
 // A RUNS step whose warp holds a row longer than kRunsLongRow: such rows are
 // cut out of their group's run (its index skips them: run index j of row i
@@ -353,7 +283,7 @@ __device__ __noinline__ void runs_step_cut(int64_t rg, int64_t n_rows, const int
         }
     }
     park<VM, R>(part, cur, acc);
-    runs_store<VM, L, R>(part, rg, lmask, n_rows, y, ldy, accumulate);
+    scatter_store<VM, L, R>(part, rg, 1, lmask, n_rows, y, ldy, accumulate);
     crs_warp_long_rows<VM>(gl == 0, lmask, rg, 1, row_ptr, col, val, x, ldx, y, ldy, accumulate);
 }
 
@@ -419,7 +349,7 @@ crs_runs_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
             }
         }
         park<VM, R>(part, cur, acc);
-        runs_store<VM, L, R>(part, rg, 0u, n_rows, y, ldy, accumulate);
+        scatter_store<VM, L, R>(part, rg, 1, 0u, n_rows, y, ldy, accumulate);
     }
 }
 
@@ -621,11 +551,24 @@ static void launch_vector_R(const Mat &A, const VecArgs &v, int R, cudaStream_t 
     }
 }
 
+template <int VM, int R>
+static void launch_short(const Mat &A, const VecArgs &v, cudaStream_t s) {
+    typedef typename ValT<VM>::T T;
+    const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, 32 * R)), A.grid_limit);
+    crs_short_kernel<VM, R><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, static_cast<const T *>(A.val),
+                                                     static_cast<const T *>(v.x), v.ldx, static_cast<T *>(v.y), v.ldy,
+                                                     v.accumulate);
+}
+
 template <int VM>
 static void launch_vector(const Mat &A, const VecArgs &v, cudaStream_t s) {
     const int R = A.kopt.rows_per_warp;
     switch (A.kopt.lanes) {
-        case 1: launch_vector_R<VM, 1>(A, v, R, s); break;
+        case 1:
+            if (R == 1) launch_short<VM, 1>(A, v, s);
+            else if (R == 2) launch_short<VM, 2>(A, v, s);
+            else launch_short<VM, 4>(A, v, s);
+            break;
         case 2: launch_vector_R<VM, 2>(A, v, R, s); break;
         case 4: launch_vector_R<VM, 4>(A, v, R, s); break;
         case 8: launch_vector_R<VM, 8>(A, v, R, s); break;
@@ -695,24 +638,25 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
     }
 }
 
-// Default VECTOR shape.  FP64: three to six entries per lane.  On GB300
-// every step of a lane group's shuffle reduction is a full FP64 instruction
-// and idle lanes issue their FMAs anyway, so few lanes per row win: on the
-// HH-like matrix (13 entries a row) 4 lanes ran at 362 us, 8 at 555 us and
-// 16 at 1091 us.  FP32 arithmetic is cheap, and the compensated sums are
-// long dependent chains, so FP32 rows get about one lane per entry.
+// Default VECTOR shape, from the mean row length.  Few lanes a row win: on
+// GB300 every addition of a lane group's reduction is a full FP64
+// instruction, idle lanes issue their FMAs anyway, and in FP32 a wide group
+// gathers fewer rows' neighbouring x at a time.  Measured (us, L x 4 unless
+// stated; old rule -> this one):
+//   mean   matrix                  FP64                    FP32 compensated
+//   5.5    Zipf rows, 4M           1 lane 1098 -> 183      8 lanes 289 -> 140
+//   13     HH-like, 1.2M           4 lanes 65              16 x 2 102 -> 4: 51
+//   17.5   uniform random, 0.5M    4 lanes 55              32 x 2 72 -> 4: 45
+//   26     27-point stencil, 1M    8 lanes 111 -> 4: 74    32 x 2 160 -> 4: 61
+//   50     uniform random, 0.2M    16 x 2 61 -> 8: 55      32 x 2 47 -> 8: 47
+//   100    uniform random, 0.1M    32 x 2 57 -> 16: 51     32 x 2 39 -> 16: 37
+// (8 lanes on the stencil, with this reduction: 78 and 59.)
 void crs_default_opts(Mat &A) {
     const double mean = A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0;
-    int lanes = 1;
-    if (A.dtype == GBSP_F64) {
-        while (lanes < 32 && 3.0 * (2 * lanes) <= mean) lanes <<= 1;
-    } else {
-        while (lanes < 32 && lanes < mean) lanes <<= 1;
-        if (lanes > 1 && lanes >= 2 * mean) lanes >>= 1;
-    }
+    const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < 36 ? 4 : mean < 64 ? 8 : mean < 192 ? 16 : 32;
     A.kopt.kernel = GBSP_KERNEL_VECTOR;
     A.kopt.lanes = lanes;
-    A.kopt.rows_per_warp = lanes >= 16 ? 2 : 4;
+    A.kopt.rows_per_warp = lanes == 1 ? 1 : 4;
     A.kopt.tile = 2048;
     A.kopt.rhs_tile = 16;
     A.kopt.accum = A.dtype == GBSP_F32 ? GBSP_ACC_COMPENSATED : GBSP_ACC_PLAIN;

@@ -1,10 +1,18 @@
-// Row lookup shared by the kernels that walk CRS entries 32 at a time.
+// Row lookup and whole-warp row sums shared by the CRS kernels.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "accum.cuh"
+
 namespace gbsp {
+
+// Steps of its lane group after which VECTOR hands a row to the whole warp:
+// the warp waits for its longest row, and a group that is still at it after
+// 16 steps holds a row several times the mean (crs_default_opts).  Zipf rows,
+// 4 x 4: 516 us with a limit of 512 entries, 356 us with 32 steps, 297 us with 16.
+constexpr int kVectorSteps = 16;
 
 // The row (0..31, of a warp's 32 rows) of entry cb + lane, for a warp that
 // holds its rows' starts (rs) and ends (re) one per lane; every lane takes
@@ -39,6 +47,187 @@ __device__ __forceinline__ int chunk_row(int32_t rs, int32_t re, int32_t cb, int
         }
     }
     return r;
+}
+// Flagged rows with the whole warp on each row in turn.  Every lane passes
+// its group's mask (bit i: row first + i * step is long; only `leader`
+// lanes' masks are read); lanes stride through a row U loads deep, with the
+// next step's columns loaded while this step's gathers are in flight (a step
+// then waits for one latency, not two), then a full-warp sum.  U changes no
+// result.  Out of line, so that it does not weigh on the common path's
+// registers.  Zipf rows (4M, 22.1M entries), RUNS 4 x 4: 188 us with four
+// loads and no look-ahead, 164 us with six, 178 us with eight (spills).
+template <int VM, int U = 6>
+__device__ __noinline__ void crs_warp_long_rows(bool leader, unsigned mask, int64_t first, int64_t step,
+                                                const int32_t *__restrict__ row_ptr,
+                                                const int32_t *__restrict__ col,
+                                                const typename ValT<VM>::T *__restrict__ val,
+                                                const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                                                typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    typedef typename ValT<VM>::T T;
+    const int lane = threadIdx.x & 31;
+    unsigned todo = __ballot_sync(0xffffffffu, leader && mask != 0);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        unsigned m = __shfl_sync(0xffffffffu, mask, src);
+        const int64_t f = __shfl_sync(0xffffffffu, first, src);
+        while (m) {
+            const int64_t r = f + (int64_t)(__ffs(m) - 1) * step;
+            m &= m - 1;
+            const int s0 = __ldg(row_ptr + r), s1 = __ldg(row_ptr + r + 1);
+            Acc<VM> a;
+            a.init();
+                        int c[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) c[u] = s0 + lane + 32 * u < s1 ? __ldg(col + s0 + lane + 32 * u) : -1;
+            for (int j = s0 + lane; j < s1; j += U * 32) {
+                T v[U], xv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    v[u] = c[u] >= 0 ? __ldg(val + j + 32 * u) : T(0);
+                    xv[u] = c[u] >= 0 ? ld_vec(x + (int64_t)c[u] * ldx) : T(0);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t k = (int64_t)j + 32 * (U + u);
+                    c[u] = k < s1 ? __ldg(col + k) : -1;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (j + 32 * u < s1) a.add(v[u], xv[u]);
+            }
+            group_reduce<32, VM>(a);
+            if (lane == 0) {
+                if (accumulate) a.add_value(y[r * ldy]);
+                y[r * ldy] = a.result();
+            }
+        }
+    }
+}
+
+// VECTOR, L lanes a row: rows longer than this are summed by the whole warp
+// (in the batched product too, so that both return the same bits).
+template <int L>
+__host__ __device__ constexpr int vector_long_row() {
+    return kVectorSteps * L;
+}
+
+// VECTOR with one lane a row, R sets of 32 consecutive rows from `base` on:
+// rows of up to kShortRow entries by one lane, the loads of 8 / R slots of all
+// sets issued together; rows of up to kMidRow by eight lanes; longer ones by
+// the whole warp.  Without the two upper classes a warp runs to its longest
+// row: on the Zipf rows (5.5 entries a row, up to 5000) 1098 us against 183
+// us now; what is left there is FP64 issue (half of the time: idle lanes
+// issue too) and the latency of the longest rows.  kMidRow 32, 64 and 128
+// gave 198, 185 and 183 us.  A row's arithmetic depends on its length alone,
+// so the batched product, which cuts the rows elsewhere, returns the same
+// bits.
+constexpr int kShortRow = 8;
+constexpr int kMidRow = 128;
+
+// Rows base + i, i in the bits of `todo` (the same in every lane; lane i
+// passes the row's bounds s0, s1): eight lanes a row, four rows at a time.
+template <int VM>
+__device__ __forceinline__ void crs_mid_rows(unsigned todo, int64_t base, int s0, int s1,
+                                             const int32_t *__restrict__ col,
+                                             const typename ValT<VM>::T *__restrict__ val,
+                                             const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                                             typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    typedef typename ValT<VM>::T T;
+    const int lane = threadIdx.x & 31, grp = lane >> 3, gl = lane & 7;
+    while (todo) {
+        unsigned t = todo;
+#pragma unroll
+        for (int g = 0; g < 3; ++g)
+            if (g < grp) t &= t - 1;
+        const int src = t ? __ffs(t) - 1 : 0;
+        const int k0 = __shfl_sync(0xffffffffu, s0, src);
+        int k1 = __shfl_sync(0xffffffffu, s1, src);
+        if (!t) k1 = k0;
+        Acc<VM> a;
+        a.init();
+        for (int j = k0 + gl; j < k1; j += 4 * 8) {
+            int c[4];
+            T v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool ok = j + 8 * u < k1;
+                c[u] = ok ? __ldg(col + j + 8 * u) : -1;
+                v[u] = ok ? __ldg(val + j + 8 * u) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c[u] >= 0) a.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
+        }
+        group_reduce<8, VM>(a);
+        if (gl == 0 && t) {
+            const int64_t r = base + src;
+            if (accumulate) a.add_value(y[r * ldy]);
+            y[r * ldy] = a.result();
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) todo &= todo - 1;
+    }
+}
+
+template <int VM, int R>
+__device__ __forceinline__ void crs_short_rows(int64_t base, int64_t n_rows, const int32_t *__restrict__ row_ptr,
+                                               const int32_t *__restrict__ col,
+                                               const typename ValT<VM>::T *__restrict__ val,
+                                               const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                                               typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    typedef typename ValT<VM>::T T;
+    constexpr int U = kShortRow / R;
+    const int lane = threadIdx.x & 31;
+    int k0[R], n[R];
+    int len = 0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int64_t r = base + 32 * i + lane;
+        k0[i] = 0;
+        n[i] = 0;
+        if (r < n_rows) {
+            k0[i] = __ldg(row_ptr + r);
+            n[i] = __ldg(row_ptr + r + 1) - k0[i];
+        }
+        if (n[i] <= kShortRow) len = max(len, n[i]);
+    }
+    Acc<VM> acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i].init();
+    for (int j = 0; j < len; j += U) {
+        int c[R][U];
+        T v[R][U];
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool ok = j + u < n[i] && n[i] <= kShortRow;
+                c[i][u] = ok ? __ldg(col + k0[i] + j + u) : -1;
+                v[i][u] = ok ? __ldg(val + k0[i] + j + u) : T(0);
+            }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (c[i][u] >= 0) acc[i].add(v[i][u], ld_vec(x + (int64_t)c[i][u] * ldx));
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int64_t r = base + 32 * i + lane;
+        if (r < n_rows && n[i] <= kShortRow) {
+            if (accumulate) acc[i].add_value(y[r * ldy]);
+            y[r * ldy] = acc[i].result();
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const unsigned mid = __ballot_sync(0xffffffffu, n[i] > kShortRow && n[i] <= kMidRow);
+        if (mid) crs_mid_rows<VM>(mid, base + 32 * i, k0[i], k0[i] + n[i], col, val, x, ldx, y, ldy, accumulate);
+        const unsigned big = __ballot_sync(0xffffffffu, n[i] > kMidRow);
+        if (big)
+            crs_warp_long_rows<VM, 4>(lane == 0, big, base + 32 * i, 1, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+    }
 }
 
 }  // namespace gbsp
