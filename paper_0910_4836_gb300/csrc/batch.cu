@@ -78,28 +78,20 @@ __device__ void batch_crs_rows(const BatchMat &m, int64_t rb, int64_t re) {
     }
 }
 
-// CRS rows with k > 1: lanes over right-hand sides (same as crs_spmm_kernel).
-template <int VM, int KT>
-__device__ void batch_crs_spmm_rows(const BatchMat &m, int64_t rb, int64_t re, int c0) {
+// CRS rows with k > 1: lanes over right-hand sides, about 32 rows a warp at
+// a time, taken by length (spmm_rows; row by row the same FMA chains as
+// crs_spmm_kernel).
+template <int VM, int W>
+__device__ void batch_crs_spmm_rows(const BatchMat &m, int64_t rb, int64_t re, int c0, uint8_t (*order)[32]) {
     typedef typename ValT<VM>::T T;
-    constexpr int G = 32 / KT;
-    const int lane = threadIdx.x & 31, grp = lane / KT, c = lane % KT, wid = threadIdx.x >> 5;
-    const int cc = c0 + c;
-    const bool active = cc < m.k;
-    const T *val = static_cast<const T *>(m.val);
-    const T *X = static_cast<const T *>(m.x);
-    T *Y = static_cast<T *>(m.y);
-    for (int64_t r = rb + (int64_t)wid * G + grp; r < re; r += (int64_t)(kBatchThreads / 32) * G) {
-        const int k0 = __ldg(m.row_ptr + r), k1 = __ldg(m.row_ptr + r + 1);
-        Acc<VM> acc;
-        acc.init();
-        for (int j = k0; j < k1; ++j) {
-            const int ci = __ldg(m.col + j);
-            const T vi = __ldg(val + j);
-            if (active) acc.add(vi, ld_vec(X + (int64_t)ci * m.ldx + cc));
-        }
-        if (active) Y[r * m.ldy + cc] = acc.result();
-    }
+    constexpr int G = 32 / W;
+    const int lane = threadIdx.x & 31, grp = lane / W, cc = c0 + lane % W, wid = threadIdx.x >> 5;
+    const bool active = grp < G && cc < m.k;
+    constexpr int rows = 32 / G * G;
+    for (int64_t r = rb + (int64_t)wid * rows; r < re; r += (int64_t)(kBatchThreads / 32) * rows)
+        spmm_rows<VM, W>(r, (int)min((int64_t)rows, re - r), active, order[wid], m.row_ptr, m.col,
+                         static_cast<const T *>(m.val), static_cast<const T *>(m.x) + cc, m.ldx,
+                         static_cast<T *>(m.y) + cc, m.ldy, 0);
 }
 
 // JDS-family rows [rb, re): one thread per row, every right-hand side of the
@@ -202,17 +194,18 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
     }
 }
 
-// Right-hand-side tiles are clamped to KTMAX, the widest tile the kernel
-// instance carries (a batch whose matrices all have k = 1 runs an instance
-// without the wide-tile code and its registers; k = 16 runs as two 8-wide
-// tiles at twice the occupancy of a 16-wide one).  The tile width never
+// Right-hand-side tiles of JDS-family items are clamped to KTMAX, the widest
+// tile the kernel instance carries (a batch without several right-hand sides
+// on such items runs an instance without the wide-tile code and its
+// registers; k = 16 runs as two 8-wide tiles at twice the occupancy of a
+// 16-wide one).  The tile width never
 // changes a result: every right-hand side is summed on its own, in the same
 // entry order.
 template <int KTMAX>
 __device__ __forceinline__ int clamp_tile(int kt) { return kt < KTMAX ? kt : KTMAX; }
 
-template <int VM, int KTMAX>
-__device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re) {
+template <int VM, int KTMAX, bool CRS1>
+__device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*order)[32]) {
     if (m.kind == KIND_JDS && m.format == GBSP_SELL) {
         int KT = 1;
         if (m.k > 1) {
@@ -234,7 +227,7 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re) {
     }
     if (m.kind == KIND_CRS) {
         if (m.k == 1) {
-            switch (m.lanes) {
+            if constexpr (CRS1) switch (m.lanes) {
                 case 1: batch_crs_rows<VM, 1>(m, rb, re); break;
                 case 2: batch_crs_rows<VM, 2>(m, rb, re); break;
                 case 4: batch_crs_rows<VM, 4>(m, rb, re); break;
@@ -242,17 +235,10 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re) {
                 case 16: batch_crs_rows<VM, 16>(m, rb, re); break;
                 default: batch_crs_rows<VM, 32>(m, rb, re); break;
             }
-        } else if constexpr (KTMAX >= 2) {
-            int KT = 2;
-            while (KT < min(m.k, m.rhs_tile > 0 ? min(m.rhs_tile, 32) : 16)) KT <<= 1;
-            KT = clamp_tile<KTMAX>(KT);
-            for (int c0 = 0; c0 < m.k; c0 += KT) {
-                if (KT == 2) batch_crs_spmm_rows<VM, 2>(m, rb, re, c0);
-                if constexpr (KTMAX >= 4) if (KT == 4) batch_crs_spmm_rows<VM, 4>(m, rb, re, c0);
-                if constexpr (KTMAX >= 8) if (KT == 8) batch_crs_spmm_rows<VM, 8>(m, rb, re, c0);
-                if constexpr (KTMAX >= 16) if (KT == 16) batch_crs_spmm_rows<VM, 16>(m, rb, re, c0);
-                if constexpr (KTMAX >= 32) if (KT >= 32) batch_crs_spmm_rows<VM, 32>(m, rb, re, c0);
-            }
+        } else {
+            with_spmm_width(spmm_width(m.k, m.rhs_tile), [&](auto W) {
+                for (int c0 = 0; c0 < m.k; c0 += W.value) batch_crs_spmm_rows<VM, W.value>(m, rb, re, c0, order);
+            });
         }
     } else {
         if (m.k == 1) {
@@ -271,12 +257,19 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re) {
     }
 }
 
-template <int KTMAX>
-__global__ void __launch_bounds__(kBatchThreads, KTMAX == 1 ? 5 : 4)
+// CTAs per SM.  The instance without several right-hand sides on JDS-family
+// items and without one on CRS items takes eight: the batch is bound by FP64
+// issue and by the latency of its gathers, and 32 registers with some spills
+// beat five or six CTAs with none (256 matrices, mixed k, FP64: 1736, 1666
+// and 1603 us for five, six and eight; one kernel with 64 registers for any
+// k > 4 took 2160 us).
+template <int KTMAX, bool CRS1>
+__global__ void __launch_bounds__(kBatchThreads, KTMAX > 1 ? 4 : CRS1 ? 5 : 8)
 batch_kernel(const BatchMat *__restrict__ mats, const BatchWork *__restrict__ work, int64_t n_work,
              int32_t *counter, const volatile int32_t *ready, int32_t *status) {
     __shared__ int64_t next[2];
     __shared__ int32_t go;
+    __shared__ uint8_t order[kBatchThreads / 32][32];
     if (threadIdx.x == 0) {
         go = 1;
         if (ready) {
@@ -307,9 +300,9 @@ batch_kernel(const BatchMat *__restrict__ mats, const BatchWork *__restrict__ wo
         if (w >= n_work) break;
         const BatchWork wk = work[w];
         const BatchMat m = mats[wk.mat];
-        if (m.vm == VM_F64) batch_item<VM_F64, KTMAX>(m, wk.rb, wk.re);
-        else if (m.vm == VM_F32C) batch_item<VM_F32C, KTMAX>(m, wk.rb, wk.re);
-        else batch_item<VM_F32, KTMAX>(m, wk.rb, wk.re);
+        if (m.vm == VM_F64) batch_item<VM_F64, KTMAX, CRS1>(m, wk.rb, wk.re, order);
+        else if (m.vm == VM_F32C) batch_item<VM_F32C, KTMAX, CRS1>(m, wk.rb, wk.re, order);
+        else batch_item<VM_F32, KTMAX, CRS1>(m, wk.rb, wk.re, order);
         if (threadIdx.x == 0) next[i ^ 1] = atomicAdd(counter, 1);
         // every thread has read next[i]; next[i ^ 1] is written and visible
         __syncthreads();
@@ -328,10 +321,20 @@ struct gbsp_batch_s {
     const BatchWork *work = nullptr;
     const int32_t *ready = nullptr;
     int grid = 0;
-    int ktmax = 1;  // widest right-hand-side tile of the kernel instance: 1, 4 or 8
+    const void *kernel = nullptr;  // the batch_kernel instance for this batch's items
 };
 
 namespace {
+
+// The kernel instance decides the registers, hence the CTAs per SM: the
+// widest tile of JDS-family items with several right-hand sides, and
+// whether any CRS item has one (CRS items with several need neither).
+const void *batch_instance(int kmax, bool crs1) {
+    if (kmax > 4) return reinterpret_cast<const void *>(batch_kernel<8, true>);
+    if (kmax > 1) return reinterpret_cast<const void *>(batch_kernel<4, true>);
+    if (crs1) return reinterpret_cast<const void *>(batch_kernel<1, true>);
+    return reinterpret_cast<const void *>(batch_kernel<1, false>);
+}
 
 constexpr int64_t kCounterBytes = 256;
 
@@ -495,18 +498,14 @@ gbsp_status gbsp_batch_create(int32_t n, const gbsp_batch_item *items, int32_t c
                                   cudaMemcpyHostToDevice, s));
     GBSP_CUDA(cudaStreamSynchronize(s));  // host vectors go out of scope
     int kmax = 1;
-    for (int32_t i = 0; i < n; ++i) kmax = std::max(kmax, (int)items[i].k);
-    // the widest tile decides the registers, hence the CTAs per SM: 48
-    // registers for 1 (5 CTAs of 256 threads), 64 for 4 and 8 (4 CTAs),
-    // about 128 for 16 (2 CTAs); wider k runs as several 8-wide tiles
-    b->ktmax = kmax == 1 ? 1 : (kmax <= 4 ? 4 : 8);
+    bool crs1 = false;
+    for (int32_t i = 0; i < n; ++i) {
+        if (items[i].A->kind != KIND_CRS) kmax = std::max(kmax, (int)items[i].k);
+        else if (items[i].k == 1) crs1 = true;
+    }
+    b->kernel = batch_instance(kmax, crs1);
     int per_sm = 0;
-    if (b->ktmax == 1)
-        GBSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<1>, kBatchThreads, 0));
-    else if (b->ktmax == 4)
-        GBSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<4>, kBatchThreads, 0));
-    else
-        GBSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<8>, kBatchThreads, 0));
+    GBSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kBatchThreads, 0));
     b->grid = (int)std::max<int64_t>(1, std::min<int64_t>(b->n_work, (int64_t)num_sms() * std::max(per_sm, 1)));
     *out = b;
     return GBSP_OK;
@@ -517,12 +516,8 @@ gbsp_status gbsp_batch_run(gbsp_batch b, int32_t *d_status, void *stream) {
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (b->n_work == 0) return GBSP_OK;
     GBSP_CUDA(cudaMemsetAsync(b->counter, 0, sizeof(int32_t), s));
-    if (b->ktmax == 1)
-        batch_kernel<1><<<b->grid, kBatchThreads, 0, s>>>(b->mats, b->work, b->n_work, b->counter, b->ready, d_status);
-    else if (b->ktmax == 4)
-        batch_kernel<4><<<b->grid, kBatchThreads, 0, s>>>(b->mats, b->work, b->n_work, b->counter, b->ready, d_status);
-    else
-        batch_kernel<8><<<b->grid, kBatchThreads, 0, s>>>(b->mats, b->work, b->n_work, b->counter, b->ready, d_status);
+    void *args[] = {&b->mats, &b->work, &b->n_work, &b->counter, &b->ready, &d_status};
+    GBSP_CUDA(cudaLaunchKernel(b->kernel, dim3((unsigned)b->grid), dim3(kBatchThreads), args, 0, s));
     GBSP_LAUNCH_CHECK("batch_kernel");
     return GBSP_OK;
 }

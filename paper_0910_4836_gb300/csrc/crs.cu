@@ -17,9 +17,9 @@
 // RUNS: as VECTOR, but a group's rows are consecutive and its lanes stride
 // through their entries as one run (below).
 //
-// SpMM: lanes over right-hand sides -- a group of KT lanes owns one row and
-// lane c accumulates column c of the RHS tile, so each entry (val, col) is
-// read once per tile and X's row slice is read as one contiguous segment.
+// SpMM: lanes over right-hand sides -- lane c of a group accumulates column
+// c of the pass, so each entry (val, col) is read once per pass and X's row
+// slice is read as one contiguous segment.
 //
 // All three run in CTAs of two warps, one CTA per two warps' worth of rows
 // (row_grid below).
@@ -353,22 +353,43 @@ crs_runs_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
     }
 }
 
-template <int VM, int KT>
-__global__ void __launch_bounds__(kThreads)
+constexpr int kRowCta = 64;  // see row_grid
+
+// SpMM: the lanes of a warp form 32 / W groups of W lanes, one lane per
+// right-hand side of the pass.  FP64: a warp takes about 16 rows and the
+// groups take them by length (spmm_rows): bound by FP64 issue (90% of it on
+// the HH-like matrix, N = 1,201,200: k = 16 487 -> 452 us, k = 5 281 -> 182
+// us, k = 3 158 -> 131 us).  Few rows a warp keep the rows that are in work at
+// one time close together: 32 instead of 16 took 540 us, X's rows leaving L2
+// before the other diagonals come back to them; fewer than 64 warps an SM
+// (more than 32 registers) cost as much as longer steps gain.  Where
+// the groups cover those rows in one round, and in FP32, which is not bound
+// by FP64 issue, a group takes one row in matrix order.
+template <int VM, int W>
+__host__ __device__ constexpr int spmm_rows_per_warp() {
+    return VM == VM_F64 && 32 / W < 16 ? 16 / (32 / W) * (32 / W) : 32 / W;
+}
+
+template <int VM, int W>
+__global__ void __launch_bounds__(kThreads, spmm_rows_per_warp<VM, W>() > 32 / W ? 8 : 0)
 crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                 const typename ValT<VM>::T *__restrict__ X, int64_t ldx,
                 typename ValT<VM>::T *__restrict__ Y, int64_t ldy, int k, int c0, int accumulate) {
     typedef typename ValT<VM>::T T;
-    constexpr int G = 32 / KT;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / KT, c = lane % KT;
-    const int cc = c0 + c;
-    const bool active = cc < k;
+    __shared__ uint8_t order[kRowCta / 32][32];
+    constexpr int G = 32 / W, RW = spmm_rows_per_warp<VM, W>();
+    const int lane = threadIdx.x & 31, grp = lane / W, cc = c0 + lane % W;
+    const bool active = grp < G && cc < k;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r = warp * G + grp; r - grp < n_rows; r += nwarp * G) {
-        if (r >= n_rows) continue;
+    if (RW > G) {
+        if (warp * RW < n_rows)
+            spmm_rows<VM, W>(warp * RW, (int)min((int64_t)RW, n_rows - warp * RW), active, order[threadIdx.x >> 5],
+                             row_ptr, col, val, X + cc, ldx, Y + cc, ldy, accumulate);
+        return;
+    }
+    for (int64_t r = warp * G + grp; r - grp < n_rows; r += ((int64_t)gridDim.x * blockDim.x >> 5) * G) {
+        if (r >= n_rows || grp >= G) continue;
         const int k0 = __ldg(row_ptr + r), k1 = __ldg(row_ptr + r + 1);
         Acc<VM> acc;
         acc.init();
@@ -522,7 +543,6 @@ static int grid_for(int64_t warps_needed) {
 // keeps the SMs full of warps with work left.  HH-like 6M, CRS vector 4 x 4:
 // 289 us against 305 us with 256-thread CTAs on a four-wave grid; Zipf
 // rows 515 against 584 us; SpMM k = 16 2489 against 2680 us.
-constexpr int kRowCta = 64;
 static int row_grid(int64_t warps_needed) {
     return (int)std::max<int64_t>(1, ceil_div(warps_needed, kRowCta / 32));
 }
@@ -602,40 +622,14 @@ static void launch_runs(const Mat &A, const VecArgs &v, cudaStream_t s) {
 template <int VM>
 static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
     typedef typename ValT<VM>::T T;
-    int kt = A.kopt.rhs_tile > 0 ? A.kopt.rhs_tile : 16;
-    kt = std::min(kt, 32);
-    // lanes per row: the power of two covering min(k, tile)
-    int cols = std::min<int>(v.k, kt);
-    int KT = 2;
-    while (KT < cols) KT <<= 1;
-    auto *val = static_cast<const T *>(A.val);
-    auto *X = static_cast<const T *>(v.x);
-    auto *Y = static_cast<T *>(v.y);
-    const int grid = row_grid(ceil_div(A.n_rows, 32 / KT));
-    for (int c0 = 0; c0 < v.k; c0 += KT) {
-        switch (KT) {
-            case 2:
-                crs_spmm_kernel<VM, 2><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, X,
-                                                                 v.ldx, Y, v.ldy, v.k, c0, v.accumulate);
-                break;
-            case 4:
-                crs_spmm_kernel<VM, 4><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, X,
-                                                                 v.ldx, Y, v.ldy, v.k, c0, v.accumulate);
-                break;
-            case 8:
-                crs_spmm_kernel<VM, 8><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, X,
-                                                                 v.ldx, Y, v.ldy, v.k, c0, v.accumulate);
-                break;
-            case 16:
-                crs_spmm_kernel<VM, 16><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, X,
-                                                                  v.ldx, Y, v.ldy, v.k, c0, v.accumulate);
-                break;
-            default:
-                crs_spmm_kernel<VM, 32><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, X,
-                                                                  v.ldx, Y, v.ldy, v.k, c0, v.accumulate);
-                break;
-        }
-    }
+    const int w = spmm_width(v.k, A.kopt.rhs_tile);
+    with_spmm_width(w, [&](auto W) {
+        const int grid = row_grid(ceil_div(A.n_rows, (int64_t)spmm_rows_per_warp<VM, W.value>()));
+        for (int c0 = 0; c0 < v.k; c0 += W.value)
+            crs_spmm_kernel<VM, W.value><<<grid, kRowCta, 0, s>>>(
+                A.n_rows, A.row_ptr, A.col, static_cast<const T *>(A.val), static_cast<const T *>(v.x), v.ldx,
+                static_cast<T *>(v.y), v.ldy, v.k, c0, v.accumulate);
+    });
 }
 
 // Default VECTOR shape, from the mean row length.  Few lanes a row win: on

@@ -230,4 +230,98 @@ __device__ __forceinline__ void crs_short_rows(int64_t base, int64_t n_rows, con
     }
 }
 
+// SpMM: lanes per row of a pass over k right-hand sides, at most `tile` (16
+// when unset) of them a pass, in passes of equal width: the widest groups
+// that leave as many groups to a warp (32 / width) as the pass's columns do.
+__host__ __device__ inline int spmm_width(int k, int tile) {
+    const int t = tile > 0 ? (tile < 32 ? tile : 32) : 16;
+    const int passes = (k + t - 1) / t;
+    return 32 / (32 / ((k + passes - 1) / passes));
+}
+
+// Calls f(Num<W>()) for the width w >= 2 of spmm_width.
+template <int N> struct Num { static constexpr int value = N; };
+template <typename F>
+__host__ __device__ __forceinline__ void with_spmm_width(int w, F f) {
+    if (w <= 2) f(Num<2>());
+    else if (w <= 3) f(Num<3>());
+    else if (w <= 4) f(Num<4>());
+    else if (w <= 5) f(Num<5>());
+    else if (w <= 6) f(Num<6>());
+    else if (w <= 8) f(Num<8>());
+    else if (w <= 10) f(Num<10>());
+    else if (w <= 16) f(Num<16>());
+    else f(Num<32>());
+}
+
+// SpMM: rows [r0, r0 + nr), nr <= 32, of one warp, whose lanes form 32 / W
+// groups of W lanes, one lane per right-hand side of the pass (X and Y point
+// at its column; idle lanes pass active = false).  The groups take one row
+// each per round, rows in order of decreasing length, so that the rows of a
+// round are about equally long: in matrix order the groups of a warp wait
+// for its longest row, and an FP64 instruction costs the same however many of
+// its lanes are active, even none.  Hence also the exact tail in FP64: with
+// four predicated slots a step the HH-like matrix took 8.7M warp-wide FMAs for
+// k = 16, with the tail 7.8M (7.6M is one full warp each).  Every row is one
+// FMA chain in entry order, whatever its round.  `order`: 32 bytes of shared
+// memory of the warp.
+template <int VM, int W>
+__device__ __forceinline__ void spmm_rows(int64_t r0, int nr, bool active, uint8_t *order,
+                                          const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                                          const typename ValT<VM>::T *__restrict__ val,
+                                          const typename ValT<VM>::T *__restrict__ X, int64_t ldx,
+                                          typename ValT<VM>::T *__restrict__ Y, int64_t ldy, int accumulate) {
+    typedef typename ValT<VM>::T T;
+    constexpr int G = 32 / W;
+    const int lane = threadIdx.x & 31, grp = lane / W;
+    // lane i: start and length of row r0 + i
+    const int s = __ldg(row_ptr + r0 + min(lane, nr));
+    const int n = lane < nr ? __ldg(row_ptr + r0 + lane + 1) - s : -1;
+    int rank = 0;
+    for (int i = 0; i < nr; ++i) {
+        const int m = __shfl_sync(0xffffffffu, n, i);
+        rank += m > n || (m == n && i < lane);
+    }
+    __syncwarp();
+    if (lane < nr) order[rank] = (uint8_t)lane;
+    __syncwarp();
+    for (int t = 0; t < nr; t += G) {
+        const int longest = __shfl_sync(0xffffffffu, n, order[t]);
+        const bool mine = active && t + grp < nr;
+        const int src = t + grp < nr ? order[t + grp] : 0;
+        const int k0 = __shfl_sync(0xffffffffu, s, src);
+        const int len = __shfl_sync(0xffffffffu, n, src);
+        Acc<VM> acc;
+        acc.init();
+        const int32_t *cp = col + k0;
+        const T *vp = val + k0;
+        // N entries of the row from j on
+        auto entries = [&](auto N, int j) {
+            int c[N.value];
+            T v[N.value];
+#pragma unroll
+            for (int u = 0; u < N.value; ++u) {
+                const bool ok = mine && j + u < len;
+                c[u] = ok ? __ldg(cp + j + u) : -1;
+                v[u] = ok ? __ldg(vp + j + u) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < N.value; ++u)
+                if (c[u] >= 0) acc.add(v[u], ld_vec(X + (int64_t)c[u] * ldx));
+        };
+        int j = 0;
+        for (; j + (VM == VM_F64 ? 4 : 1) <= longest; j += 4) entries(Num<4>(), j);
+        switch (VM == VM_F64 ? longest - j : 0) {
+            case 3: entries(Num<3>(), j); break;
+            case 2: entries(Num<2>(), j); break;
+            case 1: entries(Num<1>(), j); break;
+        }
+        if (mine) {
+            T *y = Y + (r0 + src) * ldy;
+            if (accumulate) acc.add_value(*y);
+            *y = acc.result();
+        }
+    }
+}
+
 }  // namespace gbsp
