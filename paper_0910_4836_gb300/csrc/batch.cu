@@ -148,8 +148,8 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t b = rb / 32 + wid; b * 32 < re; b += kBatchThreads / 32) {
         const int64_t r = b * 32 + lane;
-        const int32_t len = r < m.n_rows ? __ldg(m.rlen + r) : 0;
-        const int32_t width = __shfl_sync(0xffffffffu, len, 0);
+        int32_t len = r < m.n_rows ? __ldg(m.rlen + r) : 0;  // less the slots done
+        int32_t left = __shfl_sync(0xffffffffu, len, 0);
         int32_t off = __ldg(m.blk_ptr + b);  // entry offsets fit int32
         Acc<VM> acc[KT];
 #pragma unroll
@@ -164,9 +164,11 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
             v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
             off += __popc(__ballot_sync(0xffffffffu, ok));
         }
-        for (int32_t d0 = 0; d0 < width; d0 += U) {
+        // products of the first N slots in flight (the last step has fewer
+        // than U; see sell_walk)
+        auto products = [&](auto N) {
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
+            for (int j = 0; j < N.value; ++j) {
                 if (c[j] < 0) continue;
                 if (PLAIN) {
                     acc[0].add(v[j], ld_vec(x + c[j]));
@@ -177,14 +179,23 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
                         if (c0 + q < m.k) acc[q].add(v[j], ld_vec(xr + q));
                 }
             }
-            if (d0 + U >= width) break;
+        };
+        for (; left > U; left -= U) {
+            products(Num<U>());
+            len -= U;
 #pragma unroll
             for (int j = 0; j < U; ++j) {
-                const bool ok = len > d0 + U + j;
+                const bool ok = len > j;
                 c[j] = ok ? ld_stream(m.col + (off + lane)) : -1;
                 v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
                 off += __popc(__ballot_sync(0xffffffffu, ok));
             }
+        }
+        switch (left) {
+            case 1: products(Num<1>()); break;
+            case 2: products(Num<2>()); break;
+            case 3: products(Num<3>()); break;
+            case 4: products(Num<4>()); break;
         }
         if (r < m.n_rows) {
 #pragma unroll

@@ -22,10 +22,12 @@
 #include <algorithm>
 #include <atomic>
 #include <climits>
+#include <type_traits>
 #include <vector>
 
 #include "accum.cuh"
 #include "internal.cuh"
+#include "rows.cuh"
 
 namespace gbsp {
 
@@ -340,16 +342,29 @@ __global__ void __launch_bounds__(256) jds_block_kernel(JdsArgs a) {
 // 1024-row window at a time and its gathers of x stay local.  U slots per
 // step; KT right-hand sides per thread (SpMM).  Row entries are added in
 // slot order, as in every JDS-family kernel.
-template <int VM, int U, int KT, bool PLAIN>
+// EXACT: the last step forms the products of the slots that are left, instead
+// of U of which some are past the block's longest row: an FP64 instruction
+// takes its 64 cycles of a sub-partition's pipe with every lane predicated
+// off, too (HH-like, u = 4: 10% fewer).  It pays where FP64 issue or the
+// instruction count is what bounds the walk: N = 1.2M 48.4 -> 45.6 us, 3M
+// 108.2 -> 107.5, a 1000 x 1000 Laplacian 22.8 -> 18.5, FP32 compensated N =
+// 2M 59.5 -> 56.9; with vectors past L2's reach (6M), where HBM and the
+// gathers do, the plain last step is faster: 211.0 against 213.6 us.
+template <int VM, int U, int KT, bool PLAIN, bool EXACT>
 __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
     typedef typename ValT<VM>::T T;
     const T *__restrict__ val = static_cast<const T *>(a.val);
     const T *__restrict__ x = static_cast<const T *>(a.x);
     const int lane = threadIdx.x & 31;
-    const int64_t nb = ceil_div_dev(a.n_rows, 32);
+    // Rows, blocks and entry offsets all fit int32, which saves the exact last
+    // step its spills.  The plain one keeps 64-bit counters: 32-bit ones took
+    // 0.7% off at 6M rows with one matrix over and over, and added 0.4% where
+    // three matrices took turns.
+    typedef typename std::conditional<EXACT, int, int64_t>::type I;
+    const I n_rows = (I)a.n_rows, nb = (I)ceil_div_dev(a.n_rows, 32);
     const int wpc = blockDim.x >> 5;  // warps per CTA
     const int wid = threadIdx.x >> 5;
-    const int64_t ngroups = ceil_div_dev(nb, wpc);
+    const I ngroups = (nb + wpc - 1) / wpc;
     // A CTA takes wpc consecutive blocks (a group) per iteration.  Blocks are
     // sorted by length inside their window, so the warp's pick among them
     // rotates by 7 from one iteration to the next: otherwise warp 0 would
@@ -360,17 +375,17 @@ __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
     // kept as running 32-bit counters (no division in the loop).
     uint32_t rot = blockIdx.x;  // (blockIdx.x + iteration) mod gridDim.x
     int pick = wid;             // (wid + 7 iteration) mod wpc
-    for (int64_t g0 = 0; g0 < ngroups; g0 += gridDim.x) {
-        const int64_t g = g0 + rot;
-        const int64_t b = g * wpc + pick;
+    for (I g0 = 0; g0 < ngroups; g0 += gridDim.x) {
+        const I g = g0 + rot;
+        const I b = g * wpc + pick;
         rot = rot + 1 == gridDim.x ? 0u : rot + 1;
         pick += 7;
         while (pick >= wpc) pick -= wpc;
         if (g >= ngroups || b >= nb) continue;
-        const int64_t r = b * 32 + lane;
+        const I r = b * 32 + lane;
         // row lengths are read once: streamed like val / col (evict-first)
-        const int32_t len = r < a.n_rows ? ld_stream(a.rlen + r) : 0;
-        const int32_t width = __shfl_sync(0xffffffffu, len, 0);  // lane 0 holds the longest row
+        int32_t len = r < n_rows ? ld_stream(a.rlen + r) : 0;  // less the slots done
+        int32_t left = __shfl_sync(0xffffffffu, len, 0);         // lane 0 holds the longest row
         // entry offsets fit int32 (nnz < 2^31)
         int32_t off = __ldg(a.blk_ptr + b);
         Acc<VM> acc[KT];
@@ -387,9 +402,10 @@ __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
             v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
             off += __popc(__ballot_sync(0xffffffffu, ok));
         }
-        for (int32_t d0 = 0; d0 < width; d0 += U) {
+        // products of the first N slots in flight
+        auto products = [&](auto N) {
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
+            for (int j = 0; j < N.value; ++j) {
                 if (c[j] < 0) continue;
                 if (PLAIN) {
                     acc[0].add(v[j], ld_vec(x + c[j]));
@@ -400,16 +416,40 @@ __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
                         if (KT == 1 || a.c0 + q < a.k) acc[q].add(v[j], ld_vec(xr + q));
                 }
             }
-            if (d0 + U >= width) break;
+        };
+        if (EXACT) {
+            for (; left > U; left -= U) {
+                products(Num<U>());
+                len -= U;
 #pragma unroll
-            for (int j = 0; j < U; ++j) {
-                const bool ok = len > d0 + U + j;
-                c[j] = ok ? ld_stream(a.col + (off + lane)) : -1;
-                v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
-                off += __popc(__ballot_sync(0xffffffffu, ok));
+                for (int j = 0; j < U; ++j) {
+                    const bool ok = len > j;
+                    c[j] = ok ? ld_stream(a.col + (off + lane)) : -1;
+                    v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
+                    off += __popc(__ballot_sync(0xffffffffu, ok));
+                }
+            }
+            switch (left) {
+                case 1: products(Num<1>()); break;
+                case 2: products(Num<(U < 2 ? U : 2)>()); break;
+                case 3: products(Num<(U < 3 ? U : 3)>()); break;
+                case 4: products(Num<(U < 4 ? U : 4)>()); break;
+            }
+        } else {
+            const int width = left;
+            for (int d0 = 0; d0 < width; d0 += U) {
+                products(Num<U>());
+                if (d0 + U >= width) break;
+#pragma unroll
+                for (int j = 0; j < U; ++j) {
+                    const bool ok = len > d0 + U + j;
+                    c[j] = ok ? ld_stream(a.col + (off + lane)) : -1;
+                    v[j] = ok ? ld_stream(val + (off + lane)) : T(0);
+                    off += __popc(__ballot_sync(0xffffffffu, ok));
+                }
             }
         }
-        if (r < a.n_rows) {
+        if (r < n_rows) {
 #pragma unroll
             for (int q = 0; q < KT; ++q)
                 if (KT == 1 || a.c0 + q < a.k) store_row_sell<VM>(a, r, a.c0 + q, acc[q]);
@@ -420,7 +460,7 @@ __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
 
 template <int VM, int U, int KT, bool PLAIN>
 __global__ void __launch_bounds__(1024) sell_kernel(JdsArgs a) {
-    sell_walk<VM, U, KT, PLAIN>(a);
+    sell_walk<VM, U, KT, PLAIN, true>(a);
 }
 
 // The plain one-vector FP64 walk compiled for two CTAs per SM: at the same
@@ -428,9 +468,9 @@ __global__ void __launch_bounds__(1024) sell_kernel(JdsArgs a) {
 // other instances keep the kernel above: under the hint the SpMM ones would
 // spill and the FP32 ones ran 3% slower, and a hint of one CTA per SM gives
 // them 48 registers.
-template <int U>
+template <int U, bool EXACT>
 __global__ void __launch_bounds__(1024, 2) sell_kernel_f64(JdsArgs a) {
-    sell_walk<VM_F64, U, 1, true>(a);
+    sell_walk<VM_F64, U, 1, true, EXACT>(a);
 }
 
 // SELL with the banded part of x staged in shared memory.  A CTA of 32 warps
@@ -702,7 +742,10 @@ static void launch_sell_U(JdsArgs a, int KT, cudaStream_t s) {
     const bool plain = KT == 1 && !a.x_perm && a.ldx == 1 && a.c0 == 0;
     switch (KT) {
         case 1:
-            if (plain && VM == VM_F64) sell_kernel_f64<U><<<(unsigned)grid, threads, 0, s>>>(a);
+            // the line lies where y starts to be written evict-first: vectors
+            // of more than a quarter of L2
+            if (plain && VM == VM_F64 && a.y_evict_first) sell_kernel_f64<U, false><<<(unsigned)grid, threads, 0, s>>>(a);
+            else if (plain && VM == VM_F64) sell_kernel_f64<U, true><<<(unsigned)grid, threads, 0, s>>>(a);
             else if (plain) sell_kernel<VM, U, 1, true><<<(unsigned)grid, threads, 0, s>>>(a);
             else sell_kernel<VM, U, 1, false><<<(unsigned)grid, threads, 0, s>>>(a);
             break;
