@@ -5,6 +5,8 @@
 // LSD radix sort whose per-tile ranks come from warp match/ballot
 // operations in a fixed (round, warp, lane) order; integer atomics only
 // count.  So every output array is a bit-exact function of the input.
+#include <cuda_pipeline_primitives.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -270,18 +272,26 @@ gbsp_status sort_keys(uint32_t *keys, int64_t n, int bits, void *ws, cudaStream_
 
 // ------------------------------------------------------------ JDS build --
 
-__global__ void row_len_kernel(int64_t n, const int32_t *__restrict__ row_ptr, int32_t *len,
-                               int32_t *max_len) {
+// Row lengths (if `len` is given) and their maximum: one atomic per CTA, and
+// none where a longer row has been seen already (integer: the order does not
+// matter).  An atomic per warp took 41 us for 2M rows, most of it waiting for
+// the one address.
+__global__ void __launch_bounds__(256)
+row_len_kernel(int64_t n, const int32_t *__restrict__ row_ptr, int32_t *len, int32_t *max_len) {
+    __shared__ unsigned best;
+    if (threadIdx.x == 0) best = 0;
+    __syncthreads();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int32_t l = 0;
     if (i < n) {
         l = row_ptr[i + 1] - row_ptr[i];
         if (len) len[i] = l;
     }
-    // warp max then one atomic per warp (integer: order-independent)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) l = max(l, __shfl_xor_sync(0xffffffffu, l, off));
-    if ((threadIdx.x & 31) == 0 && l > 0) atomicMax(max_len, l);
+    const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)max(l, 0));
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(&best, m);
+    __syncthreads();
+    if (threadIdx.x == 0 && (int32_t)best > *reinterpret_cast<volatile int32_t *>(max_len))
+        atomicMax(max_len, (int32_t)best);
 }
 
 __global__ void len_key_kernel(int64_t n, const int32_t *__restrict__ len, int32_t max_len,
@@ -308,25 +318,84 @@ __global__ void diag_len_kernel(int64_t n, int64_t n_diag, const int32_t *__rest
 }
 
 // val_jds[jd_ptr[d] + r] = val[row_ptr[perm[r]] + d], col likewise
-// (renumbered by iperm under the symmetric permutation).
+// (renumbered by iperm under the symmetric permutation).  A thread takes a
+// permuted row's first kScatterDepth entries; the rest of a longer row, of
+// which there are few and which one thread would copy alone long after the
+// others, goes to a warp (jds_scatter_deep_kernel): Zipf rows, 1M, 2312 us with
+// a thread for each whole row, 31 + 82 us so.
+constexpr int kScatterDepth = 32;
 template <typename T>
 __global__ void jds_scatter_kernel(int64_t n, const int32_t *__restrict__ perm,
                                    const int32_t *__restrict__ iperm,
                                    const int32_t *__restrict__ row_ptr,
                                    const int32_t *__restrict__ col, const T *__restrict__ val,
                                    const int32_t *__restrict__ jd_ptr, int64_t n_diag,
-                                   int symmetric, int32_t *col_out, T *val_out, int32_t *vmap) {
+                                   int symmetric, int32_t *__restrict__ col_out, T *__restrict__ val_out,
+                                   int32_t *__restrict__ vmap) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const int32_t src = row_ptr[perm[r]];
+    const int32_t p = perm[r], src = row_ptr[p];
     // rows longer than the planned N_j (matrix changed after the plan) are cut
-    const int32_t len = (int32_t)min((int64_t)(row_ptr[perm[r] + 1] - src), n_diag);
-    for (int32_t d = 0; d < len; ++d) {
-        const int64_t dst = (int64_t)jd_ptr[d] + r;
-        const int32_t c = col[src + d];
-        col_out[dst] = symmetric ? iperm[c] : c;
-        val_out[dst] = val[src + d];
-        if (vmap) vmap[dst] = src + d;
+    const int32_t len = (int32_t)min(min((int64_t)(row_ptr[p + 1] - src), n_diag), (int64_t)kScatterDepth);
+    constexpr int U = 4;
+    for (int32_t d = 0; d < len; d += U) {
+        int32_t c[U];
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            c[u] = d + u < len ? __ldg(col + src + d + u) : -1;
+            v[u] = d + u < len ? __ldg(val + src + d + u) : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0 && symmetric) c[u] = __ldg(iperm + c[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c[u] < 0) continue;
+            const int64_t dst = (int64_t)__ldg(jd_ptr + d + u) + r;
+            col_out[dst] = c[u];
+            val_out[dst] = v[u];
+            if (vmap) vmap[dst] = src + d + u;
+        }
+    }
+}
+
+// Entries from kScatterDepth on: the rows that have any come first.
+template <typename T>
+__global__ void jds_scatter_deep_kernel(const int32_t *__restrict__ perm, const int32_t *__restrict__ iperm,
+                                        const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                                        const T *__restrict__ val, const int32_t *__restrict__ jd_ptr, int64_t n_diag,
+                                        int symmetric, int32_t *__restrict__ col_out, T *__restrict__ val_out,
+                                        int32_t *__restrict__ vmap) {
+    const int32_t rows = __ldg(jd_ptr + kScatterDepth + 1) - __ldg(jd_ptr + kScatterDepth);
+    const int lane = threadIdx.x & 31;
+    const int32_t warp = (int32_t)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int32_t nwarp = (int32_t)(((int64_t)gridDim.x * blockDim.x) >> 5);
+    for (int32_t r = warp; r < rows; r += nwarp) {
+        const int32_t p = perm[r], src = row_ptr[p];
+        const int32_t len = (int32_t)min((int64_t)(row_ptr[p + 1] - src), n_diag);
+        constexpr int U = 4;
+        for (int32_t d = kScatterDepth + lane; d < len; d += 32 * U) {
+            int32_t c[U], at[U];
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool ok = d + 32 * u < len;
+                c[u] = ok ? __ldg(col + src + d + 32 * u) : -1;
+                v[u] = ok ? __ldg(val + src + d + 32 * u) : T(0);
+                at[u] = ok ? __ldg(jd_ptr + d + 32 * u) + r : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (c[u] >= 0 && symmetric) c[u] = __ldg(iperm + c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (c[u] < 0) continue;
+                col_out[at[u]] = c[u];
+                val_out[at[u]] = v[u];
+                if (vmap) vmap[at[u]] = src + d + 32 * u;
+            }
+        }
     }
 }
 
@@ -491,34 +560,238 @@ __global__ void sell_block_nnz_kernel(int64_t n, int64_t nb, const int32_t *__re
     if ((threadIdx.x & 31) == 0 && (r >> 5) < nb) blk_nnz[r >> 5] = l;
 }
 
-// Thread per permuted row, warps aligned to 32-row blocks: slot d of the
+// Windows of up to kWindowSort rows sorted in one launch: a CTA takes one
+// window, or as many as fit its 256 threads, ranks every row by counting the
+// rows before it (longer, or equally long and earlier: the stable order by
+// decreasing length), and writes all that the radix path needs ten launches
+// for: perm, iperm, the sorted lengths and the entries of every block.
+// 2M rows in windows of 128: 26 us against 160 us.
+constexpr int kWindowSort = 1024;
+
+__global__ void __launch_bounds__(256)
+sell_window_kernel(int64_t n, int window, int windows, const int32_t *__restrict__ row_ptr, int32_t *__restrict__ perm,
+                   int32_t *__restrict__ iperm, int32_t *__restrict__ rlen, int32_t *__restrict__ blk_nnz) {
+    // key: length, then earlier rows first; distinct, so a row's rank is the
+    // number of larger keys in its window: those of its own 32 rows by
+    // comparing, those of the other 32-row parts by bisection in the part's
+    // sorted keys.  Rows past 2^20 entries do not fit a key and are compared
+    // one by one.
+    __shared__ __align__(16) int32_t key[kWindowSort], sorted[kWindowSort];
+    __shared__ int32_t sum[kWindowSort / 32];
+    const int64_t s0 = (int64_t)blockIdx.x * window * windows;
+    const int m = (int)min((int64_t)window * windows, n - s0);  // rows of this CTA
+    const int full = (m + 31) / 32 * 32;
+    bool big = false;
+    for (int i = threadIdx.x; i < full; i += 256) {
+        const int32_t l = i < m ? __ldg(row_ptr + s0 + i + 1) - __ldg(row_ptr + s0 + i) : 0;
+        key[i] = (i < m ? l << 10 : 0) | (kWindowSort - 1 - i);  // the padding comes last
+        big |= l >> 20 > 0;
+    }
+    if (threadIdx.x < kWindowSort / 32) sum[threadIdx.x] = 0;
+    const bool slow = __syncthreads_or(big);
+    for (int i = threadIdx.x; i < full; i += 256) {
+        const int32_t k = key[i];
+        int rank = i / 32 * 32;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+            const int4 o = *reinterpret_cast<const int4 *>(key + i / 32 * 32 + j);
+            rank += (o.x > k) + (o.y > k) + (o.z > k) + (o.w > k);
+        }
+        sorted[rank] = k;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < m; i += 256) {  // i: a place in its part's order
+        const int w0 = i / window * window, w1 = min(w0 + window, full);
+        int32_t k = sorted[i], l = k >> 10;
+        int rank = w0 + i % 32;
+        if (!slow) {
+            for (int p = w0; p < w1; p += 32) {
+                if (p == i / 32 * 32) continue;
+                int at = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1)
+                    if (sorted[p + at + step - 1] > k) at += step;
+                rank += at + (sorted[p + at] > k);
+            }
+            k = kWindowSort - 1 - (k & (kWindowSort - 1));  // the row
+        } else {
+            k = i;
+            l = __ldg(row_ptr + s0 + i + 1) - __ldg(row_ptr + s0 + i);
+            rank = w0;
+            for (int j = w0; j < min(w1, m); ++j) {
+                const int32_t o = __ldg(row_ptr + s0 + j + 1) - __ldg(row_ptr + s0 + j);
+                rank += o > l || (o == l && j < i);
+            }
+        }
+        perm[s0 + rank] = (int32_t)(s0 + k);
+        iperm[s0 + k] = (int32_t)(s0 + rank);
+        rlen[s0 + rank] = l;
+        atomicAdd(&sum[rank / 32], l);
+    }
+    __syncthreads();
+    if (threadIdx.x < (m + 31) / 32) blk_nnz[s0 / 32 + threadIdx.x] = sum[threadIdx.x];
+}
+
+// Slots of one 32-row block, one warp, lane = permuted row: slot d of the
 // block holds the rows with length > d, which are the block's first rows
 // (sorted), so the position of row r's slot d is
 // blk_ptr[b] + (entries of slots < d in the block) + (r mod 32).
+// The row's entry d is at src + d of `col` and `val` (global memory, or the
+// window staged in shared memory); e0: what to add to src for the value map.
+// Slots from kSellDeep on, where only a few long rows are left: while m rows
+// are, their slots are one contiguous run of m-tuples, copied 32 entries at
+// a time (Zipf rows, 1M: 766 us slot by slot, 106 us so).
+constexpr int kSellDeep = 64;
+
+template <typename T, int U>
+__device__ __forceinline__ void sell_copy_block(int32_t len, int32_t src, int32_t off, const int32_t *col, const T *val,
+                                                const int32_t *__restrict__ iperm, int symmetric, int32_t e0,
+                                                int32_t *__restrict__ col_out, T *__restrict__ val_out,
+                                                int32_t *__restrict__ vmap) {
+    const int lane = threadIdx.x & 31;
+    const int32_t width = __shfl_sync(0xffffffffu, len, 0), near = min(width, kSellDeep);
+    for (int32_t d = 0; d < near; d += U) {
+        int32_t c[U], at[U];
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = len > d + u && d + u < near;
+            c[u] = ok ? col[src + d + u] : -1;
+            v[u] = ok ? val[src + d + u] : T(0);
+            at[u] = off + lane;
+            off += __popc(__ballot_sync(0xffffffffu, ok));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (c[u] >= 0 && symmetric) c[u] = __ldg(iperm + c[u]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (c[u] < 0) continue;
+            col_out[at[u]] = c[u];
+            val_out[at[u]] = v[u];
+            if (vmap) vmap[at[u]] = e0 + src + d + u;
+        }
+    }
+    for (int32_t d = near; d < width;) {
+        const int m = __popc(__ballot_sync(0xffffffffu, len > d));
+        const int32_t until = __shfl_sync(0xffffffffu, len, m - 1), total = (until - d) * m;
+        for (int32_t t0 = 0; t0 < total; t0 += 32 * U) {
+            int32_t k[U], c[U];
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int32_t t = t0 + 32 * u + lane, dd = t / m;
+                k[u] = __shfl_sync(0xffffffffu, src, t - dd * m) + d + dd;
+                c[u] = t < total ? col[k[u]] : -1;
+                v[u] = t < total ? val[k[u]] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (c[u] >= 0 && symmetric) c[u] = __ldg(iperm + c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (c[u] < 0) continue;
+                const int32_t at = off + t0 + 32 * u + lane;
+                col_out[at] = c[u];
+                val_out[at] = v[u];
+                if (vmap) vmap[at] = e0 + k[u];
+            }
+        }
+        off += total;
+        d = until;
+    }
+}
+
+// A warp per block, rows read where they lie.
 template <typename T>
 __global__ void sell_scatter_kernel(int64_t n, const int32_t *__restrict__ perm,
                                     const int32_t *__restrict__ iperm, const int32_t *__restrict__ rlen,
                                     const int32_t *__restrict__ blk_ptr,
                                     const int32_t *__restrict__ row_ptr,
                                     const int32_t *__restrict__ col, const T *__restrict__ val,
-                                    int symmetric, int32_t *col_out, T *val_out, int32_t *vmap) {
+                                    int symmetric, int32_t *__restrict__ col_out, T *__restrict__ val_out,
+                                    int32_t *__restrict__ vmap) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const int32_t len = r < n ? rlen[r] : 0;
-    const int64_t src = r < n ? (int64_t)row_ptr[perm[r]] : 0;
-    int64_t off = (r >> 5) <= (n - 1) / 32 ? blk_ptr[r >> 5] : 0;
-    for (int32_t d = 0;; ++d) {
-        const unsigned mask = __ballot_sync(0xffffffffu, len > d);
-        if (!mask) break;
-        if (len > d) {
-            const int64_t dst = off + lane;
-            const int32_t c = col[src + d];
-            col_out[dst] = symmetric ? iperm[c] : c;
-            val_out[dst] = val[src + d];
-            if (vmap) vmap[dst] = (int32_t)(src + d);
-        }
-        off += __popc(mask);
+    if ((r & ~int64_t(31)) >= n) return;  // warp-uniform
+    const int32_t len = r < n ? rlen[r] : 0, src = r < n ? row_ptr[perm[r]] : 0;
+    sell_copy_block<T, 4>(len, src, __ldg(blk_ptr + (r >> 5)), col, val, iperm, symmetric, 0, col_out, val_out, vmap);
+}
+
+// A CTA per window: the window's rows are one contiguous piece of the CRS
+// arrays, which is staged in shared memory with coalesced copies; its blocks
+// then read rows from there.  Reading the rows in place touches a line per
+// lane, slot and array, every slot again.  HH-like, 2M rows, sigma 128,
+// symmetric: 168 us against 208 us in place; the latency of the iperm gathers
+// at 36 warps an SM bounds it now.  A window with more than `cap` entries is
+// read in place.
+constexpr int kStageWindow = 256;  // largest window that is staged
+template <typename T>
+__global__ void __launch_bounds__(256)
+sell_scatter_window_kernel(int64_t n, int window, int cap, const int32_t *__restrict__ perm,
+                           const int32_t *__restrict__ iperm, const int32_t *__restrict__ rlen,
+                           const int32_t *__restrict__ blk_ptr, const int32_t *__restrict__ row_ptr,
+                           const int32_t *__restrict__ col, const T *__restrict__ val, int symmetric,
+                           int32_t *__restrict__ col_out, T *__restrict__ val_out, int32_t *__restrict__ vmap) {
+    extern __shared__ __align__(16) unsigned char window_smem[];
+    T *sval = reinterpret_cast<T *>(window_smem);
+    int32_t *scol = reinterpret_cast<int32_t *>(sval + cap);
+    const int64_t w0 = (int64_t)blockIdx.x * window;
+    const int m = (int)min((int64_t)window, n - w0);
+    const int32_t e0 = __ldg(row_ptr + w0), cnt = __ldg(row_ptr + w0 + m) - e0;
+    const int lead = e0 & 3;  // entries staged before the window's first
+    const bool staged = lead + cnt <= cap;
+    if (staged) {
+        // 16 bytes a copy, from the boundary at or below the first entry (the
+        // arrays are aligned, see launch_sell_scatter); single entries at the end
+        constexpr int V = 16 / sizeof(T);
+        const int vfull = (lead + cnt) / V * V, cfull = (lead + cnt) / 4 * 4;
+        for (int i = threadIdx.x * V; i < vfull; i += blockDim.x * V)
+            __pipeline_memcpy_async(sval + i, val + e0 - lead + i, 16);
+        for (int i = threadIdx.x * 4; i < cfull; i += blockDim.x * 4)
+            __pipeline_memcpy_async(scol + i, col + e0 - lead + i, 16);
+        if ((int)threadIdx.x < lead + cnt - vfull)
+            __pipeline_memcpy_async(sval + vfull + threadIdx.x, val + e0 - lead + vfull + threadIdx.x, sizeof(T));
+        if ((int)threadIdx.x < lead + cnt - cfull)
+            __pipeline_memcpy_async(scol + cfull + threadIdx.x, col + e0 - lead + cfull + threadIdx.x, 4);
     }
+    __pipeline_commit();
+    // a thread per row of the window, a warp per block
+    const int i = threadIdx.x;
+    const int64_t r = w0 + i;
+    const int32_t len = i < m ? __ldg(rlen + r) : 0, src = i < m ? __ldg(row_ptr + __ldg(perm + r)) : 0;
+    const int32_t off = i < (m + 31) / 32 * 32 ? __ldg(blk_ptr + (r >> 5)) : 0;
+    __pipeline_wait_prior(0);
+    __syncthreads();
+    if (i >= (m + 31) / 32 * 32) return;
+    if (staged)
+        sell_copy_block<T, 8>(len, src - e0 + lead, off, scol, sval, iperm, symmetric, e0 - lead, col_out, val_out, vmap);
+    else
+        sell_copy_block<T, 4>(len, src, off, col, val, iperm, symmetric, 0, col_out, val_out, vmap);
+}
+
+template <typename T>
+static gbsp_status launch_sell_scatter(const Mat &A, int64_t window, int symmetric, const gbsp_jds_buffers &b,
+                                       cudaStream_t s) {
+    const int64_t n = A.n_rows;
+    // room for an eighth more entries than the mean window has, and for 2048
+    // (nine windows of FP64 an SM) in any case
+    const int64_t cap =
+        std::max<int64_t>(2048, ceil_div((int64_t)(1.125 * (double)A.nnz / (double)n * (double)window) + 64, 32) * 32);
+    const int64_t smem = cap * (int64_t)(sizeof(T) + 4);
+    const bool aligned = ((reinterpret_cast<uintptr_t>(A.col) | reinterpret_cast<uintptr_t>(A.val)) & 15) == 0;
+    if (window <= kStageWindow && smem <= 96 * 1024 && aligned) {
+        GBSP_CUDA(cudaFuncSetAttribute(sell_scatter_window_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem));
+        sell_scatter_window_kernel<T><<<(unsigned)ceil_div(n, window), (unsigned)window, (size_t)smem, s>>>(
+            n, (int)window, (int)cap, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col,
+            static_cast<const T *>(A.val), symmetric, b.col, static_cast<T *>(b.val), b.vmap);
+    } else {
+        sell_scatter_kernel<T><<<(unsigned)ceil_div(n, 256), 256, 0, s>>>(
+            n, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col, static_cast<const T *>(A.val), symmetric, b.col,
+            static_cast<T *>(b.val), b.vmap);
+    }
+    GBSP_LAUNCH_CHECK("sell_scatter_kernel");
+    return GBSP_OK;
 }
 
 // -------------------------------------------------------- paired SELL ----
@@ -656,6 +929,10 @@ static void launch_jds_scatter(const Mat &A, const int32_t *perm, const int32_t 
     jds_scatter_kernel<T><<<(unsigned)ceil_div(A.n_rows, 256), 256, 0, s>>>(
         A.n_rows, perm, iperm, A.row_ptr, A.col, static_cast<const T *>(A.val), jd_ptr, n_diag,
         symmetric, col_out, static_cast<T *>(val_out), vmap);
+    if (n_diag > kScatterDepth)
+        jds_scatter_deep_kernel<T><<<(unsigned)std::min<int64_t>(ceil_div(A.n_rows, 8), (int64_t)num_sms() * 8), 256, 0,
+                                     s>>>(perm, iperm, A.row_ptr, A.col, static_cast<const T *>(A.val), jd_ptr, n_diag,
+                                          symmetric, col_out, static_cast<T *>(val_out), vmap);
 }
 
 template <typename T>
@@ -714,8 +991,13 @@ static gbsp_status sell_build_impl(const Mat &A, const gbsp_jds_opts &o, const g
     int32_t *scan_ws = reinterpret_cast<int32_t *>(p);
     p += align256(scan_ws_bytes(nb + 1));
     int32_t *max_len_d = reinterpret_cast<int32_t *>(p);
-    GBSP_CUDA(cudaMemsetAsync(max_len_d, 0, 4, s));
-    if (n > 0) {
+    if (n > 0 && !paired && window <= kWindowSort) {
+        const int64_t windows = std::max<int64_t>(1, 256 / window);
+        sell_window_kernel<<<(unsigned)ceil_div(n, window * windows), 256, 0, s>>>(
+            n, (int)window, (int)windows, A.row_ptr, b.perm, b.iperm, b.rlen, blk_nnz);
+        GBSP_LAUNCH_CHECK("sell_window_kernel");
+    } else if (n > 0) {
+        GBSP_CUDA(cudaMemsetAsync(max_len_d, 0, 4, s));
         const unsigned gr = (unsigned)ceil_div(n, 256);
         row_len_kernel<<<gr, 256, 0, s>>>(n, A.row_ptr, len, max_len_d);
         const int lbits = bits_for((uint64_t)sz.n_diag);
@@ -752,7 +1034,9 @@ static gbsp_status sell_build_impl(const Mat &A, const gbsp_jds_opts &o, const g
         else
             sell_block_nnz_kernel<<<(unsigned)ceil_div(nb * 32, 256), 256, 0, s>>>(n, nb, b.rlen, blk_nnz);
         GBSP_LAUNCH_CHECK("sell perm / lengths");
-        st = scan_exclusive(blk_nnz, nb, b.blk_ptr, b.blk_ptr + nb, scan_ws, s);
+    }
+    if (n > 0) {
+        gbsp_status st = scan_exclusive(blk_nnz, nb, b.blk_ptr, b.blk_ptr + nb, scan_ws, s);
         if (st != GBSP_OK) return st;
         if (paired && A.dtype == GBSP_F64)
             psell_scatter_kernel<double><<<(unsigned)ceil_div(nb * 32, 256), 256, 0, s>>>(
@@ -763,14 +1047,11 @@ static gbsp_status sell_build_impl(const Mat &A, const gbsp_jds_opts &o, const g
                 n, nb, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col, static_cast<const float *>(A.val),
                 symmetric, b.col, static_cast<float *>(b.val), b.vmap);
         else if (A.dtype == GBSP_F64)
-            sell_scatter_kernel<double><<<(unsigned)ceil_div(nb * 32, 256), 256, 0, s>>>(
-                n, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col, static_cast<const double *>(A.val),
-                symmetric, b.col, static_cast<double *>(b.val), b.vmap);
+            st = launch_sell_scatter<double>(A, window, symmetric, b, s);
         else
-            sell_scatter_kernel<float><<<(unsigned)ceil_div(nb * 32, 256), 256, 0, s>>>(
-                n, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col, static_cast<const float *>(A.val),
-                symmetric, b.col, static_cast<float *>(b.val), b.vmap);
-        GBSP_LAUNCH_CHECK("sell_scatter_kernel");
+            st = launch_sell_scatter<float>(A, window, symmetric, b, s);
+        if (st != GBSP_OK) return st;
+        GBSP_LAUNCH_CHECK("psell_scatter_kernel");
     } else {
         GBSP_CUDA(cudaMemsetAsync(b.blk_ptr, 0, 4, s));
     }
