@@ -1216,28 +1216,38 @@ __global__ void transpose_fill_kernel(int64_t nnz, const int32_t *__restrict__ s
     t_col[t] = row_of[k];
 }
 
+// out[t] = val[map[t]], eight entries a thread, a CTA's 2048 next to each
+// other: map and out are read and written in whole lines, and the entries
+// that share a sector of val (neighbouring rows of one structure are
+// neighbouring entries of the other) mostly fall into one CTA's loads.
+// 27-point stencil, 26.5M entries, A^T's values: 105 us (78 us of HBM)
+// against 360 us with a thread walking each row of A^T; HH-like, 15.7M: 84
+// against 160 us.
+constexpr int kGatherPer = 8;
 template <typename T>
-__global__ void gather_values_kernel(int64_t nnz, const int32_t *__restrict__ tmap,
-                                     const T *__restrict__ val, T *__restrict__ out) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < nnz) out[t] = val[tmap[t]];
+__global__ void __launch_bounds__(256)
+gather_values_kernel(int64_t nnz, const int32_t *__restrict__ tmap,
+                     const T *__restrict__ val, T *__restrict__ out) {
+    const int64_t t0 = (int64_t)blockIdx.x * (256 * kGatherPer) + threadIdx.x;
+    int32_t k[kGatherPer];
+    T v[kGatherPer];
+#pragma unroll
+    for (int u = 0; u < kGatherPer; ++u) k[u] = t0 + 256 * u < nnz ? __ldcs(tmap + t0 + 256 * u) : -1;
+#pragma unroll
+    for (int u = 0; u < kGatherPer; ++u)
+        if (k[u] >= 0) v[u] = __ldg(val + k[u]);
+#pragma unroll
+    for (int u = 0; u < kGatherPer; ++u)
+        if (k[u] >= 0) out[t0 + 256 * u] = v[u];
 }
 
-// Value re-gathers in row order.  A thread (or, for SELL, a lane) owns one
+// JDS and SELL value re-gathers in row order.  A thread (a lane) owns one
 // stored row and walks its slots, so the source entries it reads, one CRS
 // row, are read together and each source sector is fetched once; in entry
 // order the lanes of a warp would take one 8-byte value from each of 32
-// sectors and come back for the rest of those sectors much later.
-template <typename T>
-__global__ void csr_rows_gather_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
-                                       const int32_t *__restrict__ map, const T *__restrict__ src,
-                                       T *__restrict__ dst) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rows) return;
-    const int32_t e1 = __ldg(row_ptr + r + 1);
-    for (int32_t e = __ldg(row_ptr + r); e < e1; ++e) dst[e] = src[__ldg(map + e)];
-}
-
+// sectors and come back for the rest of those sectors a diagonal later.
+// Four slots' loads in flight: 27-point stencil 145 -> 110 us (JDS), 154 ->
+// 113 us (SELL).
 // JDS storage (JDS, NBJDS, NUJDS): thread r walks the diagonals of permuted row r.
 template <typename T>
 __global__ void jds_rows_gather_kernel(int64_t n, int64_t n_diag, const int32_t *__restrict__ jd_ptr,
@@ -1245,11 +1255,24 @@ __global__ void jds_rows_gather_kernel(int64_t n, int64_t n_diag, const int32_t 
                                        T *__restrict__ dst) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    for (int64_t d = 0; d < n_diag; ++d) {
-        const int32_t p0 = __ldg(jd_ptr + d), p1 = __ldg(jd_ptr + d + 1);
-        if (p1 - p0 <= r) break;
-        const int64_t pos = p0 + r;
-        dst[pos] = src[__ldg(map + pos)];
+    constexpr int U = 4;  // diagonals whose loads are in flight together
+    for (int64_t d = 0; d < n_diag; d += U) {
+        int32_t pos[U], k[U];
+        T v[U];
+        int32_t p0 = __ldg(jd_ptr + d);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int32_t p1 = d + u < n_diag ? __ldg(jd_ptr + d + u + 1) : p0;
+            pos[u] = p1 - p0 > r ? p0 + (int32_t)r : -1;
+            k[u] = pos[u] >= 0 ? __ldcs(map + pos[u]) : 0;
+            p0 = p1;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = pos[u] >= 0 ? __ldg(src + k[u]) : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (pos[u] >= 0) dst[pos[u]] = v[u];
+        if (pos[U - 1] < 0) break;
     }
 }
 
@@ -1264,11 +1287,24 @@ __global__ void sell_rows_gather_kernel(int64_t n, int64_t nb, const int32_t *__
     const int64_t r = b * 32 + lane;
     const int32_t len = r < n ? __ldg(rlen + r) : 0;
     int64_t off = __ldg(blk_ptr + b);
-    for (int32_t d = 0;; ++d) {
-        const unsigned mask = __ballot_sync(0xffffffffu, len > d);
-        if (!mask) break;
-        if (len > d) dst[off + lane] = src[__ldg(map + off + lane)];
-        off += __popc(mask);
+    const int32_t width = __shfl_sync(0xffffffffu, len, 0);
+    constexpr int U = 4;  // slots whose loads are in flight together
+    for (int32_t d = 0; d < width; d += U) {
+        int64_t pos[U];
+        int32_t k[U];
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool ok = len > d + u;
+            pos[u] = off + lane;
+            k[u] = ok ? __ldcs(map + pos[u]) : -1;
+            off += __popc(__ballot_sync(0xffffffffu, ok));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = k[u] >= 0 ? __ldg(src + k[u]) : T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k[u] >= 0) dst[pos[u]] = v[u];
     }
 }
 
@@ -1374,7 +1410,7 @@ gbsp_status transpose_build_impl(const Mat &A, const gbsp_transpose_buffers &b, 
 gbsp_status gather_values_launch(int64_t n, const int32_t *map, const void *src, void *dst, int dtype,
                                  cudaStream_t s) {
     if (n == 0) return GBSP_OK;
-    const unsigned g = (unsigned)ceil_div(n, 256);
+    const unsigned g = (unsigned)ceil_div(n, 256 * kGatherPer);
     if (dtype == GBSP_F64)
         gather_values_kernel<double><<<g, 256, 0, s>>>(n, map, static_cast<const double *>(src),
                                                        static_cast<double *>(dst));
@@ -1386,18 +1422,7 @@ gbsp_status gather_values_launch(int64_t n, const int32_t *map, const void *src,
 }
 
 gbsp_status transpose_values_impl(const Mat &T, cudaStream_t s) {
-    if (T.nnz == 0) return GBSP_OK;
-    const unsigned g = (unsigned)ceil_div(T.n_rows, 256);
-    if (T.dtype == GBSP_F64)
-        csr_rows_gather_kernel<double><<<g, 256, 0, s>>>(T.n_rows, T.row_ptr, T.tmap,
-                                                         static_cast<const double *>(T.transpose_src->val),
-                                                         static_cast<double *>(const_cast<void *>(T.val)));
-    else
-        csr_rows_gather_kernel<float><<<g, 256, 0, s>>>(T.n_rows, T.row_ptr, T.tmap,
-                                                        static_cast<const float *>(T.transpose_src->val),
-                                                        static_cast<float *>(const_cast<void *>(T.val)));
-    GBSP_LAUNCH_CHECK("csr_rows_gather_kernel");
-    return GBSP_OK;
+    return gather_values_launch(T.nnz, T.tmap, T.transpose_src->val, const_cast<void *>(T.val), T.dtype, s);
 }
 
 }  // namespace gbsp

@@ -82,3 +82,19 @@ def test_sell_build_unaligned_arrays(dtype):
         G = CRSMatrix(torch.as_tensor(A.row_ptr).cuda(), col_d, val_d, A.n_cols).to_jds("SELL", "symmetric", window=128)
         assert np.array_equal(host(G.col), Os.col), lead
         assert np.array_equal(host(G.val), Os.val.astype(host(G.val).dtype)), lead
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("name", ROWS)
+def test_value_refresh_edges(name, dtype):
+    A = _matrix(ROWS[name])
+    M = crs(A, dtype)
+    T = M.transpose()
+    handles = [T.to_jds(f, "row_only", window=128, value_map=True) for f in ("SELL", "NUJDS")]
+    new = torch.as_tensor(S.vector(A.nnz, 8)).to(dtype).cuda()
+    M.set_values(new)
+    M.refresh_transpose_values()
+    assert torch.equal(T.val, new[T.tmap.long()])
+    for H in handles:
+        H.refresh_values(T.val)
+        assert torch.equal(H.val, T.val[H.vmap.long()]), H.fmt
