@@ -156,49 +156,68 @@ def spmv(pattern: Pattern, val: torch.Tensor, x: torch.Tensor) -> torch.Tensor:
 
 
 class PowerFunction(torch.autograd.Function):
-    """x_m = A^m x with checkpointed recomputation in the backward pass."""
+    """x_m = A^m x with checkpointed recomputation in the backward pass.
+
+    The last segment's vectors, which the backward pass needs first, are kept
+    from the forward pass instead of computed again; what neither gradient
+    needs is not computed (x_t only serve the value gradient)."""
 
     @staticmethod
     def forward(ctx, val, x, pattern: Pattern, m: int, c: int):
         cur = x.detach().contiguous()
         ckpts = [cur]
-        for t in range(1, m + 1):
-            cur = pattern.apply(val, cur)
-            if t % c == 0 and t < m:
+        t_last = (m - 1) // c * c  # the last segment's checkpoint
+        w = m - t_last
+        last = None  # row i: x_{m-1-i}
+        for t in range(m):
+            if t == t_last and w > 1 and ctx.needs_input_grad[0]:
+                last = torch.empty((w, cur.numel()), dtype=cur.dtype, device=cur.device)
+                last[w - 1].copy_(cur)
+            cur = pattern.apply(val, cur, out=last[m - 2 - t] if last is not None and t + 1 < m else None)
+            if (t + 1) % c == 0 and t + 1 < m:
                 ckpts.append(cur)
-        ctx.pattern, ctx.m, ctx.c = pattern, m, c
-        ctx.save_for_backward(val, *ckpts)
+        ctx.pattern, ctx.m, ctx.c, ctx.n_ckpts = pattern, m, c, len(ckpts)
+        ctx.save_for_backward(val, *ckpts, *(() if last is None else (last,)))
         return cur
 
     @staticmethod
     def backward(ctx, gm):
-        val, *ckpts = ctx.saved_tensors
+        val, *saved = ctx.saved_tensors
+        ckpts, kept = saved[:ctx.n_ckpts], saved[ctx.n_ckpts:]
         p, m, c = ctx.pattern, ctx.m, ctx.c
+        need_val, need_x = ctx.needs_input_grad[:2]
         n = p.n_rows
-        dev, dt = gm.device, gm.dtype
-        dval = torch.zeros(p.nnz, dtype=dt, device=dev) if ctx.needs_input_grad[0] else None
-        g = gm.contiguous()
+
+        def vectors(w):
+            return torch.empty((w, n), dtype=gm.dtype, device=gm.device)
+
+        dval = None
+        # Row i of G: g_{t1-i}, i.e. g_{t-1} = A^T g_t down the segment; row i
+        # of X: x_{t1-1-i}, recomputed from the checkpoint x_{t0}.  Rows are
+        # contiguous vectors, so every product reads and writes with unit
+        # stride; the fused dval takes the layout as strides.
+        G = vectors(m - (m - 1) // c * c)
+        G[0].copy_(gm)
         for seg in range((m - 1) // c, -1, -1):
             t0 = seg * c
             w = min(t0 + c, m) - t0
-            # X[:, i] = x_{t1-1-i}: recomputed from the checkpoint x_{t0}.
-            # Columns are contiguous vectors (column-major n x w), so every
-            # product reads and writes with unit stride; the fused dval takes
-            # the layout as strides.
-            X = torch.empty((w, n), dtype=dt, device=dev).t()
-            X[:, w - 1] = ckpts[seg]
-            for j in range(1, w):
-                p.apply(val, X[:, w - j:w - j + 1], out=X[:, w - 1 - j:w - j])
-            # G[:, i] = g_{t1-i}, i.e. g_{t-1} = A^T g_t down the segment
-            G = torch.empty((w, n), dtype=dt, device=dev).t()
-            G[:, 0] = g
             for i in range(1, w):
-                p.apply_t(val, G[:, i - 1:i], out=G[:, i:i + 1])
-            if dval is not None:
+                p.apply_t(val, G[i - 1], out=G[i])
+            if need_val:
+                if kept and t0 + w == m:
+                    X = kept[0]
+                else:
+                    X = vectors(w)
+                    X[w - 1].copy_(ckpts[seg])
+                    for j in range(1, w):
+                        p.apply(val, X[w - j], out=X[w - 1 - j])
                 # terms g_t[row] x_{t-1}[col] for t = t1, t1-1, ..., t0+1
-                p.bind(val).dval_multi(G, X, out=dval, accumulate=True)
-            g = p.apply_t(val, G[:, w - 1:w]).reshape(n)
-        return dval, (g if ctx.needs_input_grad[1] else None), None, None, None
+                dval = p.bind(val).dval_multi(G.t(), X.t(), out=dval, accumulate=dval is not None)
+            below = vectors(c if seg > 0 else 1)
+            if seg > 0 or need_x:
+                p.apply_t(val, G[w - 1], out=below[0])
+            G = below
+        return dval, (G[0] if need_x else None), None, None, None
 
 
 def power_apply(pattern: Pattern, val: torch.Tensor, x: torch.Tensor, m: int,
