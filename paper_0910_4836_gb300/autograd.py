@@ -48,6 +48,7 @@ class Pattern:
         self.forward = forward
         dummy = torch.zeros(max(self.nnz, 1), dtype=dtype, device=self.row_ptr.device)[: self.nnz]
         self.A = CRSMatrix(self.row_ptr, self.col, dummy, self.n_cols)
+        self._bound = None  # where the handle's values are, once bound
         if tiled:
             self.A.prepare_tiled(1024)
         self.F = None
@@ -67,7 +68,12 @@ class Pattern:
         """Point the CRS handle at `val`."""
         if val.dtype != self.dtype or val.numel() != self.nnz:
             raise ValueError("values do not match the pattern")
-        self.A.set_values(val.detach())
+        # No call where the handle points there already: self.A.val, which
+        # keeps its memory alive, must still be that memory too.
+        ptr = val.data_ptr()
+        if ptr != self._bound or ptr != self.A.val.data_ptr() or not val.is_contiguous():
+            self.A.set_values(val.detach())
+            self._bound = self.A.val.data_ptr()
         return self.A
 
     def forward_op(self, val: torch.Tensor):
@@ -136,7 +142,7 @@ class SpMVFunction(torch.autograd.Function):
     def forward(ctx, val, x, pattern: Pattern):
         ctx.pattern = pattern
         ctx.save_for_backward(val, x)
-        return pattern.apply(val, x.detach().contiguous())
+        return pattern.apply(val, x)
 
     @staticmethod
     def backward(ctx, gy):
@@ -145,7 +151,7 @@ class SpMVFunction(torch.autograd.Function):
         gy = gy.contiguous()
         dval = dx = None
         if ctx.needs_input_grad[0]:
-            dval = p.bind(val).dval(gy, x.detach().contiguous())
+            dval = p.bind(val).dval(gy, x)
         if ctx.needs_input_grad[1]:
             dx = p.apply_t(val, gy)
         return dval, dx, None

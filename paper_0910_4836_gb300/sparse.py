@@ -20,9 +20,12 @@ def _vp(t: torch.Tensor | None) -> ctypes.c_void_p:
     return ctypes.c_void_p(0 if t is None else t.data_ptr())
 
 
-def _stream(stream: torch.cuda.Stream | None = None) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream: torch.cuda.Stream | None = None) -> int:
+    """The stream's handle (the current device's current stream by default,
+    asked for without building a Stream object: 0.3 us instead of 3)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _need_cuda(t: torch.Tensor, name: str, dtype=None) -> torch.Tensor:
@@ -70,23 +73,42 @@ class _Product(_Handle):
         """Y = op(A) X for row-major X (n x k); a 1-D X is a single vector.
         For k >= 8 a CRS handle is the faster format (its lanes cover one
         row's right-hand sides); JDS-family handles gather k values a row."""
+        if X.dim() == 1:
+            return self._vector(X, out, accumulate, transpose, basis, stream)
         if not X.is_cuda or X.dtype != self.dtype:
             raise ValueError(f"X must be a CUDA tensor of dtype {self.dtype}")
-        if X.dim() == 1 or X.stride(-1) != 1:
+        if X.stride(-1) != 1:
             X = X.contiguous()
-        vec = X.dim() == 1
-        k = 1 if vec else X.shape[1]
+        k = X.shape[1]
         rows_in, rows_out = (self.n_rows, self.n_cols) if transpose else (self.n_cols, self.n_rows)
         if X.shape[0] != rows_in:
             raise ValueError(f"x has {X.shape[0]} rows, expected {rows_in}")
         if out is None:
-            out = (torch.zeros if accumulate else torch.empty)(
-                (rows_out,) if vec else (rows_out, k), dtype=self.dtype, device=X.device)
+            out = (torch.zeros if accumulate else torch.empty)((rows_out, k), dtype=self.dtype, device=X.device)
         elif out.shape[0] != rows_out or out.dtype != self.dtype:
             raise ValueError("out has the wrong shape or dtype")
-        L.check(L.load().gbsp_spmm(self._h, L.OP_T if transpose else L.OP_N, basis, k, _vp(X),
-                                   _ld(X), _vp(out), _ld(out), int(accumulate), _stream(stream)),
-                "gbsp_spmm")
+        L.check(L.load().gbsp_spmm(self._h, L.OP_T if transpose else L.OP_N, basis, k, X.data_ptr(), _ld(X),
+                                   out.data_ptr(), _ld(out), int(accumulate), _stream(stream)), "gbsp_spmm")
+        return out
+
+    def _vector(self, x, out, accumulate, transpose, basis, stream) -> torch.Tensor:
+        """One vector.  A small product takes about as long as this call, so
+        it does no more than the checks, one allocation and the C call."""
+        if not x.is_cuda or x.dtype != self.dtype:
+            raise ValueError(f"X must be a CUDA tensor of dtype {self.dtype}")
+        rows_in, rows_out = (self.n_rows, self.n_cols) if transpose else (self.n_cols, self.n_rows)
+        if x.shape[0] != rows_in:
+            raise ValueError(f"x has {x.shape[0]} rows, expected {rows_in}")
+        if not x.is_contiguous():
+            x = x.contiguous()
+        if out is None:
+            out = (torch.zeros if accumulate else torch.empty)(rows_out, dtype=self.dtype, device=x.device)
+        elif out.shape[0] != rows_out or out.dtype != self.dtype:
+            raise ValueError("out has the wrong shape or dtype")
+        st = L.load().gbsp_spmm(self._h, L.OP_T if transpose else L.OP_N, basis, 1, x.data_ptr(), 1, out.data_ptr(),
+                                _ld(out), 1 if accumulate else 0, _stream(stream))
+        if st:
+            L.check(st, "gbsp_spmm")
         return out
 
     def spmv(self, x: torch.Tensor, out: torch.Tensor | None = None, accumulate: bool = False,
@@ -94,7 +116,7 @@ class _Product(_Handle):
         """y = op(A) x (or y += op(A) x)."""
         if x.dim() != 1:
             raise ValueError("spmv takes a 1-D vector; use spmm for several")
-        return self.spmm(x, out, accumulate, transpose, basis, stream)
+        return self._vector(x, out, accumulate, transpose, basis, stream)
 
     def host_stage(self, transpose: bool = False, device=None) -> tuple[torch.Tensor, torch.Tensor]:
         """Device stages (input, output) for spmv_host, reusable across calls."""
@@ -294,7 +316,7 @@ class CRSMatrix(_Product):
         x = _need_cuda(x, "x", self.dtype)
         if out is None:
             out = (torch.zeros if accumulate else torch.empty)(self.nnz, dtype=self.dtype, device=g.device)
-        L.check(L.load().gbsp_dval(self._h, _vp(g), _vp(x), _vp(out), int(accumulate),
+        L.check(L.load().gbsp_dval(self._h, g.data_ptr(), x.data_ptr(), out.data_ptr(), int(accumulate),
                                    _stream(stream)), "gbsp_dval")
         return out
 
@@ -419,7 +441,9 @@ class JDSMatrix(_Product):
         self._stage = (col_st, pages)
 
     def spmv_original(self, x: torch.Tensor, out=None, accumulate=False, stream=None):
-        return self.spmv(x, out, accumulate, basis=L.BASIS_ORIGINAL, stream=stream)
+        if x.dim() != 1:
+            raise ValueError("spmv takes a 1-D vector; use spmm for several")
+        return self._vector(x, out, accumulate, False, L.BASIS_ORIGINAL, stream)
 
 
 class DIAMatrix(_Product):
