@@ -638,7 +638,7 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
 // gathers fewer rows' neighbouring x at a time.  Measured (us, L x 4 unless
 // stated; old rule -> this one):
 //   mean   matrix                  FP64                    FP32 compensated
-//   5.5    Zipf rows, 4M           1 lane 1098 -> 183      8 lanes 289 -> 140
+//   5.5    Zipf rows, 4M           1 lane 1098 -> 168      8 lanes 289 -> 136
 //   13     HH-like, 1.2M           4 lanes 65              16 x 2 102 -> 4: 51
 //   17.5   uniform random, 0.5M    4 lanes 55              32 x 2 72 -> 4: 45
 //   26     27-point stencil, 1M    8 lanes 111 -> 4: 74    32 x 2 160 -> 4: 61

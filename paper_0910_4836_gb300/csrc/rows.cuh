@@ -8,6 +8,23 @@
 
 namespace gbsp {
 
+// A compile-time count passed to a generic lambda.
+template <int N> struct Num { static constexpr int value = N; };
+
+// f(Num<n>()) for n in 1 .. M in FP64: a real branch per count, where a fixed
+// count of predicated slots would issue every FP64 instruction, with no lane
+// active, too.  In FP32 idle slots cost little: f(Num<M>()).
+template <int VM, int M, typename F>
+__device__ __forceinline__ void with_slots(int n, F f) {
+    if constexpr (VM == VM_F64 && M > 1) {
+        if (n < M) {
+            with_slots<VM, M - 1>(n, f);
+            return;
+        }
+    }
+    f(Num<M>());
+}
+
 // Steps of its lane group after which VECTOR hands a row to the whole warp:
 // the warp waits for its longest row, and a group that is still at it after
 // 16 steps holds a row several times the mean (crs_default_opts).  Zipf rows,
@@ -80,22 +97,27 @@ __device__ __noinline__ void crs_warp_long_rows(bool leader, unsigned mask, int6
                         int c[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) c[u] = s0 + lane + 32 * u < s1 ? __ldg(col + s0 + lane + 32 * u) : -1;
-            for (int j = s0 + lane; j < s1; j += U * 32) {
-                T v[U], xv[U];
+            auto entries = [&](auto N, int j) {  // N per lane from entry j + lane on
+                T v[N.value], xv[N.value];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    v[u] = c[u] >= 0 ? __ldg(val + j + 32 * u) : T(0);
+                for (int u = 0; u < N.value; ++u) {
+                    v[u] = c[u] >= 0 ? __ldg(val + j + lane + 32 * u) : T(0);
                     xv[u] = c[u] >= 0 ? ld_vec(x + (int64_t)c[u] * ldx) : T(0);
                 }
+                if (N.value == U) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int64_t k = (int64_t)j + 32 * (U + u);
-                    c[u] = k < s1 ? __ldg(col + k) : -1;
+                    for (int u = 0; u < U; ++u) {
+                        const int64_t k = (int64_t)j + lane + 32 * (U + u);
+                        c[u] = k < s1 ? __ldg(col + k) : -1;
+                    }
                 }
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (j + 32 * u < s1) a.add(v[u], xv[u]);
-            }
+                for (int u = 0; u < N.value; ++u)
+                    if (j + lane + 32 * u < s1) a.add(v[u], xv[u]);
+            };
+            int j = s0;
+            for (; j + 32 * U <= s1; j += 32 * U) entries(Num<U>(), j);
+            if (j < s1) with_slots<VM, U>((s1 - j + 31) >> 5, [&](auto N) { entries(N, j); });
             group_reduce<32, VM>(a);
             if (lane == 0) {
                 if (accumulate) a.add_value(y[r * ldy]);
@@ -116,10 +138,10 @@ __host__ __device__ constexpr int vector_long_row() {
 // rows of up to kShortRow entries by one lane, the loads of 8 / R slots of all
 // sets issued together; rows of up to kMidRow by eight lanes; longer ones by
 // the whole warp.  Without the two upper classes a warp runs to its longest
-// row: on the Zipf rows (5.5 entries a row, up to 5000) 1098 us against 183
-// us now; what is left there is FP64 issue (half of the time: idle lanes
-// issue too) and the latency of the longest rows.  kMidRow 32, 64 and 128
-// gave 198, 185 and 183 us.  A row's arithmetic depends on its length alone,
+// row: on the Zipf rows (5.5 entries a row, up to 5000) 1098 us against 168
+// us now (181 us with a fixed number of slots a step, see with_slots); what
+// is left there is FP64 issue (idle lanes issue too) and the latency of the
+// longest rows.  kMidRow 32, 64 and 128 gave 198, 185 and 183 us.  A row's arithmetic depends on its length alone,
 // so the batched product, which cuts the rows elsewhere, returns the same
 // bits.
 constexpr int kShortRow = 8;
@@ -146,19 +168,22 @@ __device__ __forceinline__ void crs_mid_rows(unsigned todo, int64_t base, int s0
         if (!t) k1 = k0;
         Acc<VM> a;
         a.init();
-        for (int j = k0 + gl; j < k1; j += 4 * 8) {
-            int c[4];
-            T v[4];
+        const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(k1 - k0));
+        for (int j0 = 0; j0 < longest; j0 += 4 * 8)
+            with_slots<VM, 4>(min((longest - j0 + 7) >> 3, 4), [&](auto N) {
+                const int j = k0 + j0 + gl;
+                int c[N.value];
+                T v[N.value];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool ok = j + 8 * u < k1;
-                c[u] = ok ? __ldg(col + j + 8 * u) : -1;
-                v[u] = ok ? __ldg(val + j + 8 * u) : T(0);
-            }
+                for (int u = 0; u < N.value; ++u) {
+                    const bool ok = j + 8 * u < k1;
+                    c[u] = ok ? __ldg(col + j + 8 * u) : -1;
+                    v[u] = ok ? __ldg(val + j + 8 * u) : T(0);
+                }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (c[u] >= 0) a.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
-        }
+                for (int u = 0; u < N.value; ++u)
+                    if (c[u] >= 0) a.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
+            });
         group_reduce<8, VM>(a);
         if (gl == 0 && t) {
             const int64_t r = base + src;
@@ -195,23 +220,25 @@ __device__ __forceinline__ void crs_short_rows(int64_t base, int64_t n_rows, con
     Acc<VM> acc[R];
 #pragma unroll
     for (int i = 0; i < R; ++i) acc[i].init();
-    for (int j = 0; j < len; j += U) {
-        int c[R][U];
-        T v[R][U];
+    const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
+    for (int j = 0; j < longest; j += U)
+        with_slots<VM, U>(min(longest - j, U), [&](auto N) {
+            int c[R][N.value];
+            T v[R][N.value];
 #pragma unroll
-        for (int i = 0; i < R; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const bool ok = j + u < n[i] && n[i] <= kShortRow;
-                c[i][u] = ok ? __ldg(col + k0[i] + j + u) : -1;
-                v[i][u] = ok ? __ldg(val + k0[i] + j + u) : T(0);
-            }
+                for (int u = 0; u < N.value; ++u) {
+                    const bool ok = j + u < n[i] && n[i] <= kShortRow;
+                    c[i][u] = ok ? __ldg(col + k0[i] + j + u) : -1;
+                    v[i][u] = ok ? __ldg(val + k0[i] + j + u) : T(0);
+                }
 #pragma unroll
-        for (int i = 0; i < R; ++i)
+            for (int i = 0; i < R; ++i)
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (c[i][u] >= 0) acc[i].add(v[i][u], ld_vec(x + (int64_t)c[i][u] * ldx));
-    }
+                for (int u = 0; u < N.value; ++u)
+                    if (c[i][u] >= 0) acc[i].add(v[i][u], ld_vec(x + (int64_t)c[i][u] * ldx));
+        });
 #pragma unroll
     for (int i = 0; i < R; ++i) {
         const int64_t r = base + 32 * i + lane;
@@ -240,7 +267,6 @@ __host__ __device__ inline int spmm_width(int k, int tile) {
 }
 
 // Calls f(Num<W>()) for the width w >= 2 of spmm_width.
-template <int N> struct Num { static constexpr int value = N; };
 template <typename F>
 __host__ __device__ __forceinline__ void with_spmm_width(int w, F f) {
     if (w <= 2) f(Num<2>());
