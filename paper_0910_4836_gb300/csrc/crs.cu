@@ -434,11 +434,13 @@ crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 //     L1TEX data-pipe wavefronts); dval is written evict-first (it is not
 //     read again here), which leaves L2 to the gathered vectors.
 //   m > 1 (crs_dval_multi_kernel): one chunk at a time, rows found by
-//     stepping forward through the row pointers in shared memory.  With
-//     the loop over t inside, several chunks in flight took 72 registers
-//     and ran slower (27-point stencil, m = 5: 287 us against 249 us); so did
-//     the shuffle-free row lookup with one or two chunks in flight and one or
-//     two steps loaded together (294-490 us against 259 us).
+//     stepping forward through the row pointers in shared memory; for m
+//     = 2 .. 6 the steps' loads are issued together.  27-point stencil
+//     against the loop over m: m = 2 176 -> 128 us, m = 5 247 -> 239, m = 6 346 ->
+//     285 (FP64 issue alone takes 86, 215 and 258); FP32 m = 5 181 -> 136.
+//     Four at a time for more steps gained nothing (m = 8 387 against 375 us).  With the loop, several chunks in flight took
+//     72 registers and ran slower (m = 5: 287 us against 249 us); so did the
+//     shuffle-free row lookup with one or two chunks in flight (294-490 us).
 constexpr int kDvalWarps = kThreads / 32;
 constexpr int kDvalU = 4;
 
@@ -483,8 +485,8 @@ crs_dval_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
+template <typename T, int M>
+__global__ void __launch_bounds__(kThreads, M == 0 ? 0 : M == 2 || M == 6 ? 6 : 4)
 crs_dval_multi_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, int m, const T *__restrict__ G, int64_t g_row,
                 int64_t g_t, const T *__restrict__ X, int64_t x_row, int64_t x_t, T *__restrict__ dval,
@@ -506,8 +508,19 @@ crs_dval_multi_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
             const int64_t row = r0 + r;
             const int64_t cj = ld_stream(col + e);
             T d = accumulate ? dval[e] : T(0);
-            for (int t = 0; t < m; ++t)
-                d = fma(__ldg(G + row * g_row + t * g_t), __ldg(X + cj * x_row + t * x_t), d);
+            const T *gp = G + row * g_row, *xp = X + cj * x_row;
+            if (M > 0) {
+                T gv[M > 0 ? M : 1], xv[M > 0 ? M : 1];
+#pragma unroll
+                for (int t = 0; t < M; ++t) {
+                    gv[t] = __ldg(gp + t * g_t);
+                    xv[t] = __ldg(xp + t * x_t);
+                }
+#pragma unroll
+                for (int t = 0; t < M; ++t) d = fma(gv[t], xv[t], d);
+            } else {
+                for (int t = 0; t < m; ++t) d = fma(__ldg(gp + t * g_t), __ldg(xp + t * x_t), d);
+            }
             dval[e] = d;
         }
     }
@@ -701,10 +714,21 @@ static void launch_dval(const Mat &A, int32_t m, const void *G, int64_t g_row, i
         crs_dval_kernel<T><<<grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, m, static_cast<const T *>(G), g_row,
                                                      g_t, static_cast<const T *>(X), x_row, x_t,
                                                      static_cast<T *>(dval), accumulate);
-    else
-        crs_dval_multi_kernel<T><<<grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, m, static_cast<const T *>(G),
-                                                           g_row, g_t, static_cast<const T *>(X), x_row, x_t,
-                                                           static_cast<T *>(dval), accumulate);
+    else {
+        auto go = [&](auto M) {
+            crs_dval_multi_kernel<T, M.value><<<grid, kThreads, 0, s>>>(
+                A.n_rows, A.row_ptr, A.col, m, static_cast<const T *>(G), g_row, g_t, static_cast<const T *>(X), x_row,
+                x_t, static_cast<T *>(dval), accumulate);
+        };
+        switch (m) {
+            case 2: go(Num<2>()); break;
+            case 3: go(Num<3>()); break;
+            case 4: go(Num<4>()); break;
+            case 5: go(Num<5>()); break;
+            case 6: go(Num<6>()); break;
+            default: go(Num<0>()); break;
+        }
+    }
 }
 
 gbsp_status crs_dval_launch(const Mat &A, int32_t m, const void *G, int64_t g_row, int64_t g_t,
