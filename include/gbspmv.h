@@ -339,17 +339,16 @@ gbsp_status gbsp_sell_stage(gbsp_handle sell, int32_t pages_per_group, int32_t m
  * paper has none).  The thread of a permuted row walks its jagged diagonals
  * one after another, so a few very long rows (heavy-tailed row lengths)
  * would serialise the whole product.  With a split, diagonals >= depth are
- * summed by a separate kernel in chunks of `chunk` diagonals -- one thread
+ * summed by blocks of their own in chunks of `chunk` diagonals -- one thread
  * per (row, chunk), so the long rows are spread over many threads -- into
  * partial sums in caller workspace, and the row walk stops at `depth` and
  * adds the row's partial sums (deterministic; the grouping of the sum
  * differs from the unsplit walk): rows with at most 8 chunks add them in
- * chunk order, longer rows in a fixed lane-strided tree.  Three launches per
- * product: the deep kernel runs on a stream of the handle (created here),
- * forked from `stream` and joined back with events, so it overlaps the walk;
- * the merge kernel follows on `stream` (capturable in a CUDA graph).  Calls
- * on one split handle must not overlap (they share the workspace and the
- * side stream).  k = 1 only (SpMM ignores the split).  depth = 0 removes the
+ * chunk order, longer rows in a fixed lane-strided tree.  Two launches per
+ * product, both on `stream` (capturable in a CUDA graph): one whose first
+ * blocks sum the deep chunks while the others walk the rows, then the merge.
+ * Calls on one split handle must not overlap (they share the workspace).
+ * k = 1 only (SpMM ignores the split).  depth = 0 removes the
  * split.
  * Workspace bytes from gbsp_jds_split_bytes; 256-byte aligned; borrowed
  * until destroy or the next gbsp_jds_split.  Synchronises `stream`. */

@@ -69,10 +69,6 @@ struct Mat {
     const int32_t *stage_col = nullptr;
     const int32_t *stage_pages = nullptr;
     int32_t stage_pages_per_group = 0;
-    // the deep kernel runs on a side stream of the handle, forked from and
-    // joined back to the caller's stream with these events
-    cudaStream_t split_side = nullptr;
-    cudaEvent_t split_fork = nullptr, split_join = nullptr;
     std::vector<int32_t> h_jd_ptr;  // host copy, read back once at build (literal launches)
 
     // transposed structure (CRS handle built by gbsp_transpose_build)

@@ -95,13 +95,13 @@ __device__ __forceinline__ void store_row_sell(const JdsArgs &a, int64_t r, int 
 // consecutive entries of one diagonal.
 // PLAIN: one vector read directly (no x permutation, unit stride).
 template <int VM, int U, int R, bool PLAIN>
-__global__ void __launch_bounds__(256) jds_row_kernel(JdsArgs a) {
+__device__ __forceinline__ void jds_row_walk(const JdsArgs &a, int64_t block, int64_t blocks) {
     typedef typename ValT<VM>::T T;
     const T *__restrict__ val = static_cast<const T *>(a.val);
     const T *__restrict__ x = static_cast<const T *>(a.x);
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = (block * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarp = (blocks * blockDim.x) >> 5;
     for (int64_t base = warp * 32 * R; base < a.n_rows; base += nwarp * 32 * R) {
         int64_t rr[R];
 #pragma unroll
@@ -165,11 +165,16 @@ __global__ void __launch_bounds__(256) jds_row_kernel(JdsArgs a) {
     }
 }
 
+template <int VM, int U, int R, bool PLAIN>
+__global__ void __launch_bounds__(256) jds_row_kernel(JdsArgs a) {
+    jds_row_walk<VM, U, R, PLAIN>(a, blockIdx.x, gridDim.x);
+}
+
 // Deep part of a split JDS walk: CTA items are (chunk k, 256 rows); thread
 // row r sums its entries in diagonals [d_begin, d_end) of chunk k, in slot
 // order, into part[offset_k + r].
 template <int VM>
-__global__ void __launch_bounds__(256) jds_deep_kernel(JdsArgs a, int64_t n_items) {
+__device__ __forceinline__ void jds_deep_items(const JdsArgs &a, int64_t n_items, int64_t block, int64_t blocks) {
     typedef typename ValT<VM>::T T;
     constexpr int W = 256;  // diagonals of jd_ptr staged in shared memory at a time
     constexpr int G = 8;    // diagonals whose loads are issued together
@@ -181,7 +186,7 @@ __global__ void __launch_bounds__(256) jds_deep_kernel(JdsArgs a, int64_t n_item
     // its diagonal offsets; its items come in increasing order, so the chunk
     // index only moves forward
     int32_t k = 0;
-    for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+    for (int64_t it = block; it < n_items; it += blocks) {
         while (k + 1 < a.split_k && __ldg(a.split_items + k + 1) <= it) ++k;
         const int4 t = __ldg(a.split_table + k);
         const int64_t r = (it - __ldg(a.split_items + k)) * 256 + threadIdx.x;
@@ -216,6 +221,20 @@ __global__ void __launch_bounds__(256) jds_deep_kernel(JdsArgs a, int64_t n_item
         }
         if (live) part[(int64_t)t.w + r] = acc;
     }
+}
+
+// A split walk in one launch: the first blocks take the deep items, which are
+// the longer chains, the others walk the rows.  Bound by the L1TEX stage of
+// the gathers; the walk's warps and the deep items' fill each other's waits.
+// Zipf rows, 4M, depth 16, chunk 64, with the merge: 129 us with the deep part
+// as a kernel of its own on a forked stream (37 registers: it held back the
+// walk's CTAs, and the fork and join cost several us), 115 us in one launch;
+// 1M 52.8 -> 45 us, FP32 2M 85 -> 57 us.  Six CTAs an SM: seven and eight spill
+// (1M: 51 us).
+template <int VM, int U, bool PLAIN>
+__global__ void __launch_bounds__(256, U <= 4 ? 6 : 2) jds_split_kernel(JdsArgs a, int64_t n_items, int deep_blocks) {
+    if ((int)blockIdx.x < deep_blocks) jds_deep_items<VM>(a, n_items, blockIdx.x, deep_blocks);
+    else jds_row_walk<VM, U, 1, PLAIN>(a, blockIdx.x - deep_blocks, gridDim.x - deep_blocks);
 }
 
 // Last step of a split walk: row r (a row deeper than the split depth)
@@ -694,7 +713,14 @@ static int row_grid(int64_t rows) {
 }
 
 template <int VM, int U>
-static void launch_row(const JdsArgs &a, int R, cudaStream_t s) {
+static void launch_row(const JdsArgs &a, int R, cudaStream_t s, int64_t items = 0) {
+    if (items > 0) {
+        const unsigned g1 = (unsigned)limit_grid(row_grid(a.n_rows), a.grid_limit);
+        const unsigned db = (unsigned)std::min<int64_t>(items, (int64_t)num_sms() * 16);
+        if (!a.x_perm && a.ldx == 1) jds_split_kernel<VM, U, true><<<db + g1, 256, 0, s>>>(a, items, (int)db);
+        else jds_split_kernel<VM, U, false><<<db + g1, 256, 0, s>>>(a, items, (int)db);
+        return;
+    }
     const unsigned g4 = (unsigned)limit_grid(row_grid(ceil_div(a.n_rows, 4)), a.grid_limit);
     const unsigned g2 = (unsigned)limit_grid(row_grid(ceil_div(a.n_rows, 2)), a.grid_limit);
     const unsigned g1 = (unsigned)limit_grid(row_grid(a.n_rows), a.grid_limit);
@@ -887,8 +913,8 @@ static gbsp_status launch_family(const Mat &A, JdsArgs a, cudaStream_t s) {
     const int u = fmt == GBSP_NUJDS ? A.unroll : 1;
     const int R = A.kopt.rows_per_warp > 1 ? A.kopt.rows_per_warp : 1;  // rows per thread
     if (A.split_k > 0) {
-        // deep diagonals (chunk partial sums), the walk that stops at the
-        // split depth, then the merge of the two for the deep rows
+        // deep diagonals (chunk partial sums) and the walk that stops at the
+        // split depth in one launch, then the merge of the two for the deep rows
         a.d_limit = A.split_depth;
         a.split_k = A.split_k;
         a.split_table = A.split_table;
@@ -896,20 +922,14 @@ static gbsp_status launch_family(const Mat &A, JdsArgs a, cudaStream_t s) {
         a.split_part = A.split_part;
         a.split_shallow = A.split_shallow;
         a.split_rows = A.split_rows;
-        // fork: the deep kernel on the side stream, overlapping the walk
-        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(A.split_items_total, (int64_t)num_sms() * 16));
-        GBSP_CUDA(cudaEventRecord(A.split_fork, s));
-        GBSP_CUDA(cudaStreamWaitEvent(A.split_side, A.split_fork, 0));
-        jds_deep_kernel<VM><<<(unsigned)grid, 256, 0, A.split_side>>>(a, A.split_items_total);
-        GBSP_CUDA(cudaEventRecord(A.split_join, A.split_side));
     }
-    if (u <= 1) launch_row<VM, 1>(a, R, s);
-    else if (u <= 2) launch_row<VM, 2>(a, R, s);
-    else if (u <= 4) launch_row<VM, 4>(a, R, s);
-    else if (u <= 8) launch_row<VM, 8>(a, std::min(R, 2), s);
-    else launch_row<VM, 16>(a, 1, s);
+    const int64_t items = A.split_k > 0 ? A.split_items_total : 0;
+    if (u <= 1) launch_row<VM, 1>(a, R, s, items);
+    else if (u <= 2) launch_row<VM, 2>(a, R, s, items);
+    else if (u <= 4) launch_row<VM, 4>(a, R, s, items);
+    else if (u <= 8) launch_row<VM, 8>(a, std::min(R, 2), s, items);
+    else launch_row<VM, 16>(a, 1, s, items);
     if (A.split_k > 0) {
-        GBSP_CUDA(cudaStreamWaitEvent(s, A.split_join, 0));  // join
         const int64_t work = std::max<int64_t>(A.split_wide_rows * 32, A.split_rows - A.split_wide_rows);
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(work, 256), (int64_t)num_sms() * 8));
         jds_split_merge_kernel<VM><<<(unsigned)grid, 256, 0, s>>>(a, A.split_wide_rows);
@@ -1014,11 +1034,6 @@ gbsp_status jds_split_impl(Mat &A, int32_t depth, int32_t chunk, void *ws, int64
     int4 *dt = reinterpret_cast<int4 *>(p);
     int32_t *di = reinterpret_cast<int32_t *>(p + 16 * t.size());
     const int64_t po = ((16 * (int64_t)t.size() + 4 * (int64_t)it.size()) + 255) & ~int64_t(255);
-    if (!A.split_side) {
-        GBSP_CUDA(cudaStreamCreateWithFlags(&A.split_side, cudaStreamNonBlocking));
-        GBSP_CUDA(cudaEventCreateWithFlags(&A.split_fork, cudaEventDisableTiming));
-        GBSP_CUDA(cudaEventCreateWithFlags(&A.split_join, cudaEventDisableTiming));
-    }
     GBSP_CUDA(cudaMemcpyAsync(dt, t.data(), 16 * t.size(), cudaMemcpyHostToDevice, s));
     GBSP_CUDA(cudaMemcpyAsync(di, it.data(), 4 * it.size(), cudaMemcpyHostToDevice, s));
     GBSP_CUDA(cudaStreamSynchronize(s));

@@ -1,0 +1,48 @@
+"""The split JDS walk with few and with many chunks (more than a CTA counts at
+once), every unroll depth, both bases, strided vectors: integer data, where any
+summation order gives the oracle's bits."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from gpu_util import crs, dev, host
+from paper_0910_4836_gb300 import synth as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    import paper_0910_4836_gb300 as g
+    g.build()
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("perm", ["symmetric", "row_only"])
+def test_split_walk_chunks(perm, dtype):
+    n = 3001
+    lens = S.randint(5, 1, np.arange(n), 0, 12).astype(np.int64)
+    lens[::37] = S.randint(5, 2, np.arange(lens[::37].size), 13, 90)
+    lens[[5, 700, 2999]] = (1500, 1499, 600)
+    row_ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(lens, out=row_ptr[1:])
+    nnz = int(row_ptr[-1])
+    A = S.CRS(n, n, row_ptr.astype(np.int32), S.randint(3, 1, np.arange(nnz), 0, n - 1).astype(np.int32),
+              (np.arange(nnz) % 9 - 4).astype(np.float64))
+    x = S.int_vector(n, 3, 8)
+    y0 = S.int_vector(n, 4, 50)
+    ref = O.crs_spmv(A, x)
+    xd, yd = dev(x, dtype), dev(y0, dtype)
+    X2 = torch.stack([xd.flip(0), xd], 1)
+    for unroll in (1, 2, 4, 8, 16):
+        J = crs(A, dtype).to_jds("NUJDS", perm, unroll=unroll)
+        for depth, chunk in ((16, 64), (2, 4), (12, 1), (89, 500), (1499, 7)):
+            J.split(depth, chunk)
+            assert np.array_equal(host(J.spmv_original(xd)), ref), (unroll, depth, chunk)
+            assert np.array_equal(host(J.spmv_original(xd, out=yd.clone(), accumulate=True)), ref + y0)
+            xp = J.permute(xd) if perm == "symmetric" else xd
+            assert np.array_equal(host(J.permute(J.spmv(xp), back=True)), ref), (unroll, depth, chunk)
+            Y2 = torch.zeros((n, 2), dtype=dtype, device="cuda")
+            J.spmm(X2[:, 1:], out=Y2[:, :1], basis=1)
+            assert np.array_equal(host(Y2[:, 0]), ref), (unroll, depth, chunk)
