@@ -128,7 +128,8 @@ typedef enum { GBSP_ACC_PLAIN = 0, GBSP_ACC_COMPENSATED = 1 } gbsp_accum;
  * longest row; rows longer than 64 entries are cut out of the runs and
  * summed by the whole warp.  Suits irregular row lengths; lanes in
  * {1, 2, 4, 8}, rows_per_warp in {4, 8} and at least `lanes`.  AUTO picks
- * VECTOR from the row-length mean. */
+ * VECTOR from the row-length mean and the type; with `lanes` given alone,
+ * rows picked that way are picked again for those lanes. */
 typedef enum {
     GBSP_KERNEL_AUTO = 0,
     GBSP_KERNEL_VECTOR = 1,

@@ -161,9 +161,18 @@ gbsp_status gbsp_set_kernel(gbsp_handle h, const gbsp_kernel_opts *o) {
         // every field of the pair is RUNS's own: never a VECTOR leftover
         h->kopt.lanes = o->lanes ? o->lanes : 4;
         h->kopt.rows_per_warp = o->rows_per_warp ? o->rows_per_warp : (h->kopt.lanes > 4 ? 8 : 4);
+        h->default_rows = false;
     } else {
         if (o->lanes != 0) h->kopt.lanes = o->lanes;
-        if (o->rows_per_warp != 0) h->kopt.rows_per_warp = o->rows_per_warp;
+        if (o->rows_per_warp != 0) {
+            h->kopt.rows_per_warp = o->rows_per_warp;
+            h->default_rows = false;
+        } else if (o->lanes != 0 && h->default_rows) {
+            // the default's rows belong to the default's lanes: with 1 or 2
+            // rows a group, other widths run up to 1.6x longer (8 lanes on
+            // the 27-point stencil: 125 us against 78)
+            h->kopt.rows_per_warp = o->lanes == 1 ? 1 : 4;
+        }
     }
     if (o->rhs_tile != 0) h->kopt.rhs_tile = o->rhs_tile;
     h->kopt.accum = o->accum;

@@ -654,16 +654,26 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
 //   5.5    Zipf rows, 4M           1 lane 1098 -> 168      8 lanes 289 -> 136
 //   13     HH-like, 1.2M           4 lanes 65              16 x 2 102 -> 4: 51
 //   17.5   uniform random, 0.5M    4 lanes 55              32 x 2 72 -> 4: 45
-//   26     27-point stencil, 1M    8 lanes 111 -> 4: 74    32 x 2 160 -> 4: 61
+//   26     27-point stencil, 1M    8 lanes 111 -> 4 x 2: 69  32 x 2 160 -> 8: 57
+//   26     uniform random, 0.4M    4 lanes 61 -> 4 x 2: 58 4 lanes 53 -> 8: 45
 //   50     uniform random, 0.2M    16 x 2 61 -> 8: 55      32 x 2 47 -> 8: 47
 //   100    uniform random, 0.1M    32 x 2 57 -> 16: 51     32 x 2 39 -> 16: 37
-// (8 lanes on the stencil, with this reduction: 78 and 59.)
+// Two lines inside the 4-lane range, 4 x 4 on their other side:
+//   FP64 from 24 entries a row, two rows a group: a group's rows then end
+//   too far apart for four to pay.  4 x 4 / 4 x 2: HH-like, 13: 62 / 75;
+//   random, 18.5: 47.3 / 47.2, 21.5: 49.4 / 49.6, 32: 55.7 / 53.5; stencil,
+//   60^3: 20.7 / 16.8, 100^3: 72.3 / 68.8 (8 x 4: 77.8, though 49 at 32).
+//   FP32 from 20, eight lanes: the compensated chains halve.  4 x 4 / 8 x 4:
+//   HH-like, 13: 47.7 / 51.4; random, 18.5: 41.2 / 37.0, 21.5: 43.7 / 38.3,
+//   32: 49.5 / 43.1; stencil 59.4 / 57.4 (plain sums 61.7 / 55.0).
 void crs_default_opts(Mat &A) {
     const double mean = A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0;
-    const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < 36 ? 4 : mean < 64 ? 8 : mean < 192 ? 16 : 32;
+    const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < (A.dtype == GBSP_F64 ? 36 : 20) ? 4 : mean < 64 ? 8
+                      : mean < 192 ? 16 : 32;
     A.kopt.kernel = GBSP_KERNEL_VECTOR;
     A.kopt.lanes = lanes;
-    A.kopt.rows_per_warp = lanes == 1 ? 1 : 4;
+    A.kopt.rows_per_warp = lanes == 1 ? 1 : lanes == 4 && mean >= 24 ? 2 : 4;
+    A.default_rows = A.kind == KIND_CRS;
     A.kopt.tile = 2048;
     A.kopt.rhs_tile = 16;
     A.kopt.accum = A.dtype == GBSP_F32 ? GBSP_ACC_COMPENSATED : GBSP_ACC_PLAIN;

@@ -27,6 +27,7 @@ struct Mat {
 
     // kernel options
     gbsp_kernel_opts kopt{};
+    bool default_rows = false;  // kopt.rows_per_warp is crs_default_opts' choice for kopt.lanes
 
     // TILED CRS tile table (first row of every tile, then one int4 per tile)
     const int32_t *tile_rows = nullptr;

@@ -35,6 +35,7 @@ static void apply(Mat &A, const Cand &c) {
     const int accum = A.kopt.accum;
     A.kopt = c.k;
     A.kopt.accum = accum;
+    A.default_rows = false;
     if (A.kind == KIND_JDS) {
         A.format = c.format;
         if (c.block > 0) A.block = c.block;
