@@ -779,9 +779,9 @@ static gbsp_status launch_sell_scatter(const Mat &A, int64_t window, int symmetr
         std::max<int64_t>(2048, ceil_div((int64_t)(1.125 * (double)A.nnz / (double)n * (double)window) + 64, 32) * 32);
     const int64_t smem = cap * (int64_t)(sizeof(T) + 4);
     const bool aligned = ((reinterpret_cast<uintptr_t>(A.col) | reinterpret_cast<uintptr_t>(A.val)) & 15) == 0;
-    if (window <= kStageWindow && smem <= 96 * 1024 && aligned) {
-        GBSP_CUDA(cudaFuncSetAttribute(sell_scatter_window_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
+    constexpr int kStageBytes = 96 * 1024;
+    if (window <= kStageWindow && smem <= kStageBytes && aligned) {
+        GBSP_SMEM_LIMIT(sell_scatter_window_kernel<T>, kStageBytes);
         sell_scatter_window_kernel<T><<<(unsigned)ceil_div(n, window), (unsigned)window, (size_t)smem, s>>>(
             n, (int)window, (int)cap, b.perm, b.iperm, b.rlen, b.blk_ptr, A.row_ptr, A.col,
             static_cast<const T *>(A.val), symmetric, b.col, static_cast<T *>(b.val), b.vmap);
@@ -949,17 +949,18 @@ static gbsp_status relayout_blocked(const Mat &J, int64_t block, int format, con
     }
     // SOJDS: slots per row <= n_diag; shared memory per warp = n_diag * (T + 9)
     const int64_t slots = std::max<int64_t>(J.n_diag, 1);
+    constexpr size_t kSojdsBytes = 200 * 1024;
     int warps = 4;
     size_t smem = 0;
     for (; warps >= 1; warps >>= 1) {
         smem = (size_t)warps * slots * (sizeof(T) + 4 + 4 + 1) + 64;
-        if (smem <= 200 * 1024) break;
+        if (smem <= kSojdsBytes) break;
     }
     if (warps < 1) {
-        set_error("SOJDS: rows longer than %lld entries are not supported", (long long)(200 * 1024 / (sizeof(T) + 9)));
+        set_error("SOJDS: rows longer than %lld entries are not supported", (long long)(kSojdsBytes / (sizeof(T) + 9)));
         return GBSP_ERR_UNSUPPORTED;
     }
-    GBSP_CUDA(cudaFuncSetAttribute(sojds_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GBSP_SMEM_LIMIT(sojds_kernel<T>, kSojdsBytes);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(nb, warps), (int64_t)num_sms() * 8));
     sojds_kernel<T><<<(unsigned)grid, warps * 32, smem, s>>>(J.n_rows, J.n_diag, block, nb, J.jd_ptr,
                                                              J.blk_ptr, col_in,

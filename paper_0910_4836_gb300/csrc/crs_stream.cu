@@ -334,7 +334,7 @@ gbsp_status crs_prepare_tiles(Mat &A, int32_t tile, int32_t *table, cudaStream_t
 template <int VM, int T, int S>
 static gbsp_status launch_stream_T(const Mat &A, const VecArgs &v, cudaStream_t st) {
     typedef typename ValT<VM>::T V;
-    const size_t smem = sizeof(StreamSmem<VM, T, S>);
+    constexpr size_t smem = sizeof(StreamSmem<VM, T, S>);
     // the attribute belongs to the kernel on one device: set it once per
     // device (it is cheap, and allowed during stream capture, so a device
     // index out of the table's range simply sets it on every launch)
@@ -343,9 +343,7 @@ static gbsp_status launch_stream_T(const Mat &A, const VecArgs &v, cudaStream_t 
     GBSP_CUDA(cudaGetDevice(&dev));
     const bool tracked = dev >= 0 && dev < kStreamMaxDevices;
     if (!tracked || !configured[dev].load()) {
-        cudaError_t e = cudaFuncSetAttribute(crs_stream_kernel<VM, T, S>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return cuda_status(e, "cudaFuncSetAttribute(crs_stream_kernel)");
+        GBSP_SMEM_LIMIT((crs_stream_kernel<VM, T, S>), smem);
         if (tracked) configured[dev].store(1);
     }
     int per_sm = 0;

@@ -426,10 +426,10 @@ extern "C" gbsp_status gbsp_stage_sweep(const double *d_b, int64_t len_b, double
     if (reinterpret_cast<uintptr_t>(d_b) & 15) return arg_error("gbsp_stage_sweep: B must be 16-byte aligned");
     const int grid = num_sms();
     if (n_out < grid) return arg_error("gbsp_stage_sweep: out needs one double per SM");
-    const int smem = SW_BUFS * SW_CHUNK;
+    constexpr int smem = SW_BUFS * SW_CHUNK;
     // the attribute belongs to the kernel on one device: set it on every
     // call (cheap; a per-device flag would need the device-index table)
-    GBSP_CUDA(cudaFuncSetAttribute(stage_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    GBSP_SMEM_LIMIT(stage_sweep_kernel, smem);
     stage_sweep_kernel<<<grid, 256, smem, static_cast<cudaStream_t>(stream)>>>(d_b, len_b, d_out, d_status);
     GBSP_LAUNCH_CHECK("stage_sweep_kernel");
     return GBSP_OK;

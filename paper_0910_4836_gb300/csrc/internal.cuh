@@ -95,6 +95,20 @@ gbsp_status cuda_status(cudaError_t e, const char *what);
         if (e__ != cudaSuccess) return gbsp::cuda_status(e__, what);     \
     } while (0)
 
+// Most x a CTA of the staged SELL walk holds in shared memory: two CTAs per
+// SM share about 228 KB.
+constexpr int kStagedBytes = 112 * 1024;
+
+// Allows a kernel `bytes` of dynamic shared memory.  The attribute belongs to
+// the kernel on the device, for every host thread, so `bytes` is a constant,
+// the most that any launch takes: with the size of the matrix at hand, a
+// thread with a smaller one lowers it between another's call and its launch.
+#define GBSP_SMEM_LIMIT(kernel, bytes)                                                            \
+    do {                                                                                          \
+        constexpr int limit__ = (int)(bytes);                                                     \
+        GBSP_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit__)); \
+    } while (0)
+
 inline gbsp_status arg_error(const char *msg) {
     set_error("%s", msg);
     return GBSP_ERR_ARG;

@@ -822,19 +822,16 @@ static gbsp_status launch_sell_staged_U(const Mat &A, JdsArgs a, cudaStream_t s)
     typedef typename ValT<VM>::T T;
     const int P = A.stage_pages_per_group;
     const int smem = P * kStagePage * (int)sizeof(T);
-    // largest dynamic shared memory set so far for this kernel, per device
-    static std::atomic<int> configured[kMaxDevices];
+    // the kernel's attributes, set once per device (two threads that both
+    // find them unset write the same values)
+    static std::atomic<bool> configured[kMaxDevices];
     int dev = 0;
     GBSP_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices || smem > configured[dev].load()) {
-        GBSP_CUDA(cudaFuncSetAttribute(sell_staged_kernel<VM, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    if (dev < 0 || dev >= kMaxDevices || !configured[dev].load()) {
+        GBSP_SMEM_LIMIT((sell_staged_kernel<VM, U>), kStagedBytes);
         GBSP_CUDA(cudaFuncSetAttribute(sell_staged_kernel<VM, U>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        100));
-        if (dev >= 0 && dev < kMaxDevices) {
-            int cur = configured[dev].load();
-            while (cur < smem && !configured[dev].compare_exchange_weak(cur, smem)) {
-            }
-        }
+        if (dev >= 0 && dev < kMaxDevices) configured[dev].store(true);
     }
     const int64_t ngroups = ceil_div(ceil_div(a.n_rows, 32), 32);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ngroups, (int64_t)num_sms() * 2));

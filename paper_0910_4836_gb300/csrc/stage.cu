@@ -105,9 +105,7 @@ __global__ void stage_encode_kernel(int64_t nb, const int32_t *__restrict__ blk_
 }
 
 int max_pages_for(int dtype) {
-    // two CTAs per SM share about 228 KB of shared memory
-    const int per_cta = 112 * 1024;
-    return std::min(kMaxPages, per_cta / (kPage * (dtype == GBSP_F64 ? 8 : 4)));
+    return std::min(kMaxPages, kStagedBytes / (kPage * (dtype == GBSP_F64 ? 8 : 4)));
 }
 
 }  // namespace

@@ -336,6 +336,10 @@ struct SplitPlan {
     int64_t bytes() const { return 256 + rec_bytes + count_bytes + scan_bytes; }
 };
 
+// Dynamic shared memory of split_kernel and bucket_kernel.
+static constexpr int split_smem_bytes(int buckets) { return (kSplitWarps * ((buckets + 1) / 2) + buckets) * 4; }
+static constexpr int bucket_smem_bytes(int width) { return 8 * width + 4 * kRound; }
+
 static int64_t align256(int64_t b) { return (b + 255) & ~int64_t(255); }
 
 static int bits_for(uint64_t maxv) {
@@ -394,14 +398,14 @@ static gbsp_status split_build(const Mat &A, const gbsp_transpose_buffers &b, cu
     GBSP_LAUNCH_CHECK("split_count_kernel");
     gbsp_status st = scan_exclusive(counts, p.buckets * p.tiles, counts, nullptr, scan_ws, s);
     if (st != GBSP_OK) return st;
-    const int smem = (kSplitWarps * ((p.buckets + 1) / 2) + p.buckets) * 4;
-    GBSP_CUDA(cudaFuncSetAttribute(split_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const int smem = split_smem_bytes(p.buckets);
+    GBSP_SMEM_LIMIT(split_kernel<T>, split_smem_bytes(kMaxBuckets));
     split_kernel<T><<<(unsigned)p.tiles, kSplitThreads, smem, s>>>(A.nnz, p.width, p.magic, p.bits, p.buckets, p.tiles,
                                                                    p.seg, A.col, row_of, static_cast<const T *>(A.val),
                                                                    counts, rec);
     GBSP_LAUNCH_CHECK("split_kernel");
-    const int bsmem = 8 * p.width + 4 * kRound;
-    GBSP_CUDA(cudaFuncSetAttribute(bucket_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
+    const int bsmem = bucket_smem_bytes(p.width);
+    GBSP_SMEM_LIMIT(bucket_kernel<T>, bucket_smem_bytes(kMaxWidth));
     bucket_kernel<T><<<(unsigned)p.buckets, kBucketThreads, bsmem, s>>>(A.n_cols, A.nnz, p.width, p.bits, p.buckets,
                                                                         p.tiles, counts, rec, b.t_row_ptr, b.t_col,
                                                                         static_cast<T *>(b.t_val), b.tmap);
