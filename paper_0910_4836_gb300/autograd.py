@@ -74,6 +74,9 @@ class Pattern:
         if ptr != self._bound or ptr != self.A.val.data_ptr() or not val.is_contiguous():
             self.A.set_values(val.detach())
             self._bound = self.A.val.data_ptr()
+            # what the other handles hold was gathered from memory that is no
+            # longer kept alive here: its address and version may come again
+            self._fkey = self._akey = None
         return self.A
 
     def forward_op(self, val: torch.Tensor):
