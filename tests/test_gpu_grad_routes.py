@@ -92,3 +92,66 @@ def test_handle_pointed_elsewhere_between_calls():
     dx, = torch.autograd.grad(spmv(P, val, x), x, dev(g))
     ref, s = _dx(A, v, g)
     assert np.all(np.abs(host(dx) - ref) <= 1e-14 * s + 1e-300)
+
+
+M, N = 20, 50_000
+
+
+def _power_pattern():
+    A = S.hh_like(N, 97)
+    val = dev(A.val / 64)
+    return A, _pattern(A), val
+
+
+@pytest.mark.parametrize("checkpoint", [1, 2, 5, 7, 12, 20, 30])
+def test_power_memory(checkpoint):
+    """Between forward and backward a call holds y and at most twice its
+    checkpoints, x among them, but x alone with checkpoint >= m; two calls in
+    one graph hold twice that, and no_grad holds y alone."""
+    from paper_0910_4836_gb300.autograd import power_apply
+    _, P, val = _power_pattern()
+    x = dev(S.vector(N, 98)).requires_grad_()
+    val.requires_grad_()
+    power_apply(P, val, x, 2, 1)
+    vector = N * 8 + 2048  # the allocator's rounding
+    held = 0 if checkpoint >= M else 2 * -(-M // checkpoint) - 1
+    for calls, grad in ((1, True), (2, True), (1, False)):
+        torch.cuda.synchronize()
+        before = torch.cuda.memory_allocated()
+        with torch.set_grad_enabled(grad):
+            ys = [power_apply(P, val, x, M, checkpoint) for _ in range(calls)]
+        assert torch.cuda.memory_allocated() - before <= calls * (1 + (held if grad else 0)) * vector
+        del ys
+
+
+@pytest.mark.parametrize("checkpoint", [2, 5, 20])
+def test_power_peak(checkpoint):
+    """The backward pass takes three segments, the value gradient and dx
+    beyond what the checkpoints hold."""
+    from paper_0910_4836_gb300.autograd import power_apply
+    A, P, val = _power_pattern()
+    x, g = dev(S.vector(N, 98)).requires_grad_(), dev(S.vector(N, 99))
+    val.requires_grad_()
+    torch.autograd.grad(power_apply(P, val, x, M, checkpoint), (val, x), g)
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    torch.cuda.reset_peak_memory_stats()
+    torch.autograd.grad(power_apply(P, val, x, M, checkpoint), (val, x), g)
+    peak = torch.cuda.max_memory_allocated() - before - A.nnz * 8
+    assert peak <= (3 * checkpoint + -(-M // checkpoint) + 1) * (N * 8 + 2048)
+
+
+@pytest.mark.parametrize("checkpoint", [1, 3, 5, 20])
+@pytest.mark.parametrize("needs", ["values", "x"])
+def test_power_one_gradient(needs, checkpoint):
+    """A gradient asked for alone has the bits it has beside the other."""
+    from paper_0910_4836_gb300.autograd import power_apply
+    _, P, val = _power_pattern()
+    g, xv = dev(S.vector(N, 99)), dev(S.vector(N, 98))
+    both = [val.clone().requires_grad_(), xv.clone().requires_grad_()]
+    ref = torch.autograd.grad(power_apply(P, *both, M, checkpoint), both, g)
+    at = 0 if needs == "values" else 1
+    one = [val, xv]
+    one[at] = one[at].clone().requires_grad_()
+    got, = torch.autograd.grad(power_apply(P, *one, M, checkpoint), one[at], g)
+    assert torch.equal(got, ref[at])
