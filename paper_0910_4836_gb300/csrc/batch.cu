@@ -27,7 +27,7 @@ struct BatchMat {
     int32_t k;         // right-hand sides
     int32_t lanes, rows, rhs_tile, unroll;
     int32_t block;     // RBJDS / SOJDS block
-    int32_t pad;
+    int32_t cut;       // CRS, k = 1: crs_row_cut
     int64_t n_rows, n_diag;
     const int32_t *row_ptr, *col, *jd_ptr, *blk_ptr, *rlen;
     const void *val;
@@ -66,7 +66,7 @@ __device__ void batch_crs_rows(const BatchMat &m, int64_t rb, int64_t re) {
             k0 = __ldg(m.row_ptr + r);
             k1 = __ldg(m.row_ptr + r + 1);
         }
-        const unsigned lmask = k1 - k0 > vector_long_row<L>() ? 1u : 0u;
+        const unsigned lmask = k1 - k0 > m.cut ? 1u : 0u;
         if (lmask) k1 = k0;
         Acc<VM> acc;
         acc.init();
@@ -379,6 +379,7 @@ gbsp_status make_work(int32_t n, const gbsp_batch_item *items, int32_t chunk, cu
         m.k = it.k;
         m.lanes = A.kopt.lanes > 0 ? A.kopt.lanes : 4;
         m.rows = A.kopt.rows_per_warp;
+        m.cut = A.kind == KIND_CRS ? crs_row_cut(A) : 0;
         m.rhs_tile = A.kopt.rhs_tile;
         m.unroll = A.unroll;
         m.block = A.built_block > 0 ? A.built_block : 1;

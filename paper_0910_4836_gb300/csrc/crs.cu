@@ -105,13 +105,14 @@ __device__ __forceinline__ void vector_sums(Acc<VM> (&acc)[R], const int (&k0)[R
     }
 }
 
-// A VECTOR step whose warp holds a row longer than vector_long_row: such
+// A VECTOR step whose warp holds a row longer than `cut` (crs_row_cut): such
 // rows are left out of the groups' loops and summed afterwards by the whole
 // warp.  Out of line, so that the common step keeps its registers and code
 // (with the cut in the common step the 4 x 4 shape took 76 us instead of 65 us
 // on the HH-like matrix of N = 1,201,200).
 template <int VM, int L, int R>
-__device__ __noinline__ void vector_step_cut(int64_t first, int64_t n_rows, const int32_t *__restrict__ row_ptr,
+__device__ __noinline__ void vector_step_cut(int cut, int64_t first, int64_t n_rows,
+                                             const int32_t *__restrict__ row_ptr,
                                              const int32_t *__restrict__ col,
                                              const typename ValT<VM>::T *__restrict__ val,
                                              const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
@@ -129,7 +130,7 @@ __device__ __noinline__ void vector_step_cut(int64_t first, int64_t n_rows, cons
             k0[i] = __ldg(row_ptr + r);
             k1[i] = __ldg(row_ptr + r + 1);
         }
-        if (k1[i] - k0[i] > vector_long_row<L>()) {
+        if (k1[i] - k0[i] > cut) {
             lmask |= 1u << i;
             k1[i] = k0[i];
         }
@@ -147,7 +148,7 @@ __device__ __noinline__ void vector_step_cut(int64_t first, int64_t n_rows, cons
 // call to the long-row step raised some shapes to 60.
 template <int VM, int L, int R>
 __global__ void __launch_bounds__(kThreads, R == 4 ? 5 : 6)
-crs_vector_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
+crs_vector_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
                   const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                   const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
                   typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
@@ -170,8 +171,8 @@ crs_vector_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
             }
             len = max(len, k1[i] - k0[i]);
         }
-        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)vector_long_row<L>()) {
-            vector_step_cut<VM, L, R>(base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)cut) {
+            vector_step_cut<VM, L, R>(cut, base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
             continue;
         }
         Acc<VM> acc[R];
@@ -565,20 +566,21 @@ static void launch_vector_R(const Mat &A, const VecArgs &v, int R, cudaStream_t 
     typedef typename ValT<VM>::T T;
     const int64_t rw = (32 / L) * R;
     const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, rw)), A.grid_limit);
+    const int cut = crs_row_cut(A);
     auto *val = static_cast<const T *>(A.val);
     auto *x = static_cast<const T *>(v.x);
     auto *y = static_cast<T *>(v.y);
     switch (R) {
         case 1:
-            crs_vector_kernel<VM, L, 1><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, x,
+            crs_vector_kernel<VM, L, 1><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
                                                                   v.ldx, y, v.ldy, v.accumulate);
             break;
         case 2:
-            crs_vector_kernel<VM, L, 2><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, x,
+            crs_vector_kernel<VM, L, 2><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
                                                                   v.ldx, y, v.ldy, v.accumulate);
             break;
         default:
-            crs_vector_kernel<VM, L, 4><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, val, x,
+            crs_vector_kernel<VM, L, 4><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
                                                                   v.ldx, y, v.ldy, v.accumulate);
             break;
     }
@@ -666,8 +668,17 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
 //   FP32 from 20, eight lanes: the compensated chains halve.  4 x 4 / 8 x 4:
 //   HH-like, 13: 47.7 / 51.4; random, 18.5: 41.2 / 37.0, 21.5: 43.7 / 38.3,
 //   32: 49.5 / 43.1; stencil 59.4 / 57.4 (plain sums 61.7 / 55.0).
+static double row_mean(const Mat &A) { return A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0; }
+
+int crs_row_cut(const Mat &A) {
+    const int L = A.kopt.lanes;
+    double cut = 16.0 * L;
+    if (L < 32) cut = std::max(cut, (L <= 4 ? 3 : 2) * row_mean(A));
+    return (int)std::min(cut, 1e9);
+}
+
 void crs_default_opts(Mat &A) {
-    const double mean = A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0;
+    const double mean = row_mean(A);
     const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < (A.dtype == GBSP_F64 ? 36 : 20) ? 4 : mean < 64 ? 8
                       : mean < 192 ? 16 : 32;
     A.kopt.kernel = GBSP_KERNEL_VECTOR;

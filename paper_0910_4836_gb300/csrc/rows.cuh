@@ -25,12 +25,6 @@ __device__ __forceinline__ void with_slots(int n, F f) {
     f(Num<M>());
 }
 
-// Steps of its lane group after which VECTOR hands a row to the whole warp:
-// the warp waits for its longest row, and a group that is still at it after
-// 16 steps holds a row several times the mean (crs_default_opts).  Zipf rows,
-// 4 x 4: 516 us with a limit of 512 entries, 356 us with 32 steps, 297 us with 16.
-constexpr int kVectorSteps = 16;
-
 // The row (0..31, of a warp's 32 rows) of entry cb + lane, for a warp that
 // holds its rows' starts (rs) and ends (re) one per lane; every lane takes
 // part.  An entry belongs to the last nonempty row starting at or before
@@ -125,13 +119,6 @@ __device__ __noinline__ void crs_warp_long_rows(bool leader, unsigned mask, int6
             }
         }
     }
-}
-
-// VECTOR, L lanes a row: rows longer than this are summed by the whole warp
-// (in the batched product too, so that both return the same bits).
-template <int L>
-__host__ __device__ constexpr int vector_long_row() {
-    return kVectorSteps * L;
 }
 
 // VECTOR with one lane a row, R sets of 32 consecutive rows from `base` on:
