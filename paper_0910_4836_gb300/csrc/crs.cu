@@ -668,6 +668,11 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
 //   FP32 from 20, eight lanes: the compensated chains halve.  4 x 4 / 8 x 4:
 //   HH-like, 13: 47.7 / 51.4; random, 18.5: 41.2 / 37.0, 21.5: 43.7 / 38.3,
 //   32: 49.5 / 43.1; stencil 59.4 / 57.4 (plain sums 61.7 / 55.0).
+// FP32 on long rows, columns at random, is bound by the loads a row has in
+// flight (8M entries, 8 / 16 / 32 lanes; banded in brackets): uniform 1..127:
+// 41 / 35 / 33 (23.6 / 23.1 / 23.9), log-normal of mean 60: 45 / 41 / 38 (33 /
+// 32 / 32), rows of 100: 37 / 32 / 29 (17.0 / 16.7 / 18.9), of 150: 27 / 31 /
+// 23.5 (23.6 / 16.9 / 16.1): 16 lanes from 55 and 32 from 120.
 static double row_mean(const Mat &A) { return A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0; }
 
 int crs_row_cut(const Mat &A) {
@@ -679,8 +684,9 @@ int crs_row_cut(const Mat &A) {
 
 void crs_default_opts(Mat &A) {
     const double mean = row_mean(A);
-    const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < (A.dtype == GBSP_F64 ? 36 : 20) ? 4 : mean < 64 ? 8
-                      : mean < 192 ? 16 : 32;
+    const bool f64 = A.dtype == GBSP_F64;
+    const int lanes = mean < 6 ? 1 : mean < 12 ? 2 : mean < (f64 ? 36 : 20) ? 4 : mean < (f64 ? 64 : 55) ? 8
+                      : mean < (f64 ? 192 : 120) ? 16 : 32;
     A.kopt.kernel = GBSP_KERNEL_VECTOR;
     A.kopt.lanes = lanes;
     A.kopt.rows_per_warp = lanes == 1 ? 1 : lanes == 4 && mean >= 24 ? 2 : 4;

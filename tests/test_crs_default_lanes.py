@@ -1,0 +1,27 @@
+"""Default lanes of long rows at the limits of the mean row length, in both
+types.  Host logic: handles over placeholder addresses."""
+import ctypes
+
+import pytest
+
+from paper_0910_4836_gb300 import _lib
+
+P = ctypes.c_void_p(256)  # never dereferenced on the host
+
+
+def shape(n_rows, nnz, dtype):
+    """(lanes, rows) of a new handle."""
+    h, o = ctypes.c_void_p(), _lib.KernelOpts()
+    assert _lib.load().gbsp_crs_create(n_rows, 64, nnz, P, P, P, dtype, ctypes.byref(h)) == 0
+    try:
+        assert _lib.load().gbsp_get_kernel(h, ctypes.byref(o)) == 0
+        return o.lanes, o.rows_per_warp
+    finally:
+        assert _lib.load().gbsp_destroy(h) == 0
+
+
+@pytest.mark.parametrize("mean,f64,f32", [(54, 8, 8), (55, 8, 16), (63, 8, 16), (119, 16, 16), (120, 16, 32),
+                                          (191, 16, 32)])
+def test_long_rows(mean, f64, f32):
+    assert shape(64, 64 * mean, 0) == (f64, 4)
+    assert shape(64, 64 * mean, 1) == (f32, 4)
