@@ -114,8 +114,10 @@ typedef enum { GBSP_ACC_PLAIN = 0, GBSP_ACC_COMPENSATED = 1 } gbsp_accum;
 
 /* CRS kernel choice.  VECTOR: `lanes` threads of a warp per row, each warp
  * working on `rows_per_warp` rows at a time (lanes * rows in flight); rows
- * of more than 16 * lanes entries are summed by the whole warp, and with one
- * lane a row those of 9 to 128 entries by eight lanes.
+ * of more than 16 * lanes entries and far above the mean (three times it for
+ * lanes <= 4, twice for 8 and 16) are summed by the whole warp.  With one lane
+ * a row, those of more than 8 entries (12 with rows_per_warp 2 or 4; twice the
+ * mean where that is 7 to 16) by eight lanes, of more than 128 by the warp.
  * TILED: rows grouped into tiles of `tile` merge items (rows + entries);
  * a persistent CTA streams its tiles' val, col and row_ptr slices into
  * shared memory with bulk asynchronous copies (a producer warp, mbarrier

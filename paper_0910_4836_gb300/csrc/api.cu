@@ -171,7 +171,7 @@ gbsp_status gbsp_set_kernel(gbsp_handle h, const gbsp_kernel_opts *o) {
             // the default's rows belong to the default's lanes: with 1 or 2
             // rows a group, other widths run up to 1.6x longer (8 lanes on
             // the 27-point stencil: 125 us against 78)
-            h->kopt.rows_per_warp = o->lanes == 1 ? 1 : 4;
+            h->kopt.rows_per_warp = crs_default_rows(*h);
         }
     }
     if (o->rhs_tile != 0) h->kopt.rhs_tile = o->rhs_tile;

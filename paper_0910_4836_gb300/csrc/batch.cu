@@ -56,7 +56,7 @@ __device__ void batch_crs_rows(const BatchMat &m, int64_t rb, int64_t re) {
     T *y = static_cast<T *>(m.y);
     if (L == 1) {
         for (int64_t base = rb + (int64_t)wid * 32; base < re; base += kBatchThreads)
-            crs_short_rows<VM, 1>(base, re, m.row_ptr, m.col, val, x, m.ldx, y, m.ldy, 0);
+            crs_short_rows<VM, 0>(m.cut, base, re, m.row_ptr, m.col, val, x, m.ldx, y, m.ldy, 0);
         return;
     }
     for (int64_t base = rb + (int64_t)wid * G; base < re; base += (int64_t)(kBatchThreads / 32) * G) {

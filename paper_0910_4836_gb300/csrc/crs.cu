@@ -9,10 +9,10 @@
 // butterfly of warp shuffles; when a group holds as many rows as it has
 // lanes, by a reduce-scatter that leaves each lane one row's total (same
 // tree, fewer FP64 additions: on GB300 each one is a full-rate-limited FP64
-// instruction).  Rows of more than 16 L entries are cut out of their group's
-// loop and summed by the whole warp afterwards.  With one lane a row
-// (crs_short_rows) rows are sorted into three classes by length: one lane,
-// eight lanes, the whole warp.
+// instruction).  Rows far longer than the others (crs_row_cut) are cut out of
+// their group's loop and summed by the whole warp afterwards.  With one lane
+// a row (crs_short_rows) rows are sorted into three classes by length: one
+// lane, eight lanes, the whole warp.
 //
 // RUNS: as VECTOR, but a group's rows are consecutive and its lanes stride
 // through their entries as one run (below).
@@ -172,7 +172,11 @@ crs_vector_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
             len = max(len, k1[i] - k0[i]);
         }
         if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)cut) {
-            vector_step_cut<VM, L, R>(cut, base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+            if constexpr (L == 1)
+                short_rows_cut<VM, kShortRows>(cut, base, min(base + RW, n_rows), row_ptr, col, val, x, ldx, y, ldy,
+                                               accumulate);
+            else
+                vector_step_cut<VM, L, R>(cut, base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
             continue;
         }
         Acc<VM> acc[R];
@@ -181,17 +185,54 @@ crs_vector_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
     }
 }
 
-// VECTOR with one lane a row (short rows).
-template <int VM, int R>
-__global__ void __launch_bounds__(kThreads, R == 1 ? 6 : 5)
-crs_short_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
+// VECTOR with one lane a row, one or two sets of 32 consecutive rows a warp
+// (four: crs_vector_kernel).  With one set, rows of every class are expected
+// and taken in line.  With two, a step whose rows are all short has registers
+// of its own (40, 48 warps an SM), two slots of both sets at a time.  One set
+// / two, FP64: Zipf rows, 4M, 170 / 196 us; the remainder of a hybrid matrix
+// (6M rows, 5.0 entries a row, at most 17) 158 / 125 us; rows of U{1..5} 40 /
+// 34 us; 5-point Laplacian 1000 x 1000 16.9 / 15.2 us.
+template <int VM, int R, int CUT>
+__global__ void __launch_bounds__(kThreads, 6)
+crs_short_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
                  const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                  const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
                  typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t base = warp * 32 * R; base < n_rows; base += nwarp * 32 * R)
-        crs_short_rows<VM, R>(base, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+    for (int64_t base = warp * 32 * R; base < n_rows; base += nwarp * 32 * R) {
+        if (R == 1) {
+            crs_short_rows<VM, CUT>(cut, base, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+            continue;
+        }
+        const int64_t first = base + (threadIdx.x & 31);
+        int k0[R], n[R], len = 0;
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            k0[i] = 0;
+            n[i] = 0;
+            if (first + 32 * i < n_rows) {
+                k0[i] = __ldg(row_ptr + first + 32 * i);
+                n[i] = __ldg(row_ptr + first + 32 * i + 1) - k0[i];
+            }
+            len = max(len, n[i]);
+        }
+        const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
+        if (longest > (CUT > 0 ? CUT : cut)) {
+            short_rows_cut<VM, CUT>(cut, base, min(base + 32 * R, n_rows), row_ptr, col, val, x, ldx, y, ldy, accumulate);
+            continue;
+        }
+        Acc<VM> acc[R];
+        lane_sums<VM, R, 2>(acc, k0, n, col, val, x, ldx, longest);
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const int64_t r = first + 32 * i;
+            if (r < n_rows) {
+                if (accumulate) acc[i].add_value(y[r * ldy]);
+                y[r * ldy] = acc[i].result();
+            }
+        }
+    }
 }
 
 // Park a lane's running sum in its row's slot.  Indices are compile-time
@@ -561,38 +602,29 @@ static int row_grid(int64_t warps_needed) {
     return (int)std::max<int64_t>(1, ceil_div(warps_needed, kRowCta / 32));
 }
 
-template <int VM, int L>
-static void launch_vector_R(const Mat &A, const VecArgs &v, int R, cudaStream_t s) {
+template <int VM, int L, int R>
+static void launch_vector_R(const Mat &A, const VecArgs &v, cudaStream_t s) {
     typedef typename ValT<VM>::T T;
-    const int64_t rw = (32 / L) * R;
-    const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, rw)), A.grid_limit);
-    const int cut = crs_row_cut(A);
-    auto *val = static_cast<const T *>(A.val);
-    auto *x = static_cast<const T *>(v.x);
-    auto *y = static_cast<T *>(v.y);
-    switch (R) {
-        case 1:
-            crs_vector_kernel<VM, L, 1><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
-                                                                  v.ldx, y, v.ldy, v.accumulate);
-            break;
-        case 2:
-            crs_vector_kernel<VM, L, 2><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
-                                                                  v.ldx, y, v.ldy, v.accumulate);
-            break;
-        default:
-            crs_vector_kernel<VM, L, 4><<<grid, kRowCta, 0, s>>>(cut, A.n_rows, A.row_ptr, A.col, val, x,
-                                                                  v.ldx, y, v.ldy, v.accumulate);
-            break;
-    }
+    const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, (32 / L) * R)), A.grid_limit);
+    crs_vector_kernel<VM, L, R><<<grid, kRowCta, 0, s>>>(crs_row_cut(A), A.n_rows, A.row_ptr, A.col,
+                                                         static_cast<const T *>(A.val), static_cast<const T *>(v.x),
+                                                         v.ldx, static_cast<T *>(v.y), v.ldy, v.accumulate);
 }
 
-template <int VM, int R>
+template <int VM, int L>
+static void launch_vector_L(const Mat &A, const VecArgs &v, int R, cudaStream_t s) {
+    if (R == 1) launch_vector_R<VM, L, 1>(A, v, s);
+    else if (R == 2) launch_vector_R<VM, L, 2>(A, v, s);
+    else launch_vector_R<VM, L, 4>(A, v, s);
+}
+
+template <int VM, int R, int CUT>
 static void launch_short(const Mat &A, const VecArgs &v, cudaStream_t s) {
     typedef typename ValT<VM>::T T;
     const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, 32 * R)), A.grid_limit);
-    crs_short_kernel<VM, R><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, static_cast<const T *>(A.val),
-                                                     static_cast<const T *>(v.x), v.ldx, static_cast<T *>(v.y), v.ldy,
-                                                     v.accumulate);
+    crs_short_kernel<VM, R, CUT><<<grid, kRowCta, 0, s>>>(crs_row_cut(A), A.n_rows, A.row_ptr, A.col,
+                                                     static_cast<const T *>(A.val), static_cast<const T *>(v.x),
+                                                     v.ldx, static_cast<T *>(v.y), v.ldy, v.accumulate);
 }
 
 template <int VM>
@@ -600,15 +632,17 @@ static void launch_vector(const Mat &A, const VecArgs &v, cudaStream_t s) {
     const int R = A.kopt.rows_per_warp;
     switch (A.kopt.lanes) {
         case 1:
-            if (R == 1) launch_short<VM, 1>(A, v, s);
-            else if (R == 2) launch_short<VM, 2>(A, v, s);
-            else launch_short<VM, 4>(A, v, s);
+            // a cut of its own (lanes = 1 asked for on longer rows): two sets
+            if (crs_row_cut(A) > kShortRows) launch_short<VM, 2, 0>(A, v, s);
+            else if (R == 1) launch_short<VM, 1, kShortRow>(A, v, s);
+            else if (R == 2) launch_short<VM, 2, kShortRows>(A, v, s);
+            else launch_vector_R<VM, 1, 4>(A, v, s);
             break;
-        case 2: launch_vector_R<VM, 2>(A, v, R, s); break;
-        case 4: launch_vector_R<VM, 4>(A, v, R, s); break;
-        case 8: launch_vector_R<VM, 8>(A, v, R, s); break;
-        case 16: launch_vector_R<VM, 16>(A, v, R, s); break;
-        default: launch_vector_R<VM, 32>(A, v, R, s); break;
+        case 2: launch_vector_L<VM, 2>(A, v, R, s); break;
+        case 4: launch_vector_L<VM, 4>(A, v, R, s); break;
+        case 8: launch_vector_L<VM, 8>(A, v, R, s); break;
+        case 16: launch_vector_L<VM, 16>(A, v, R, s); break;
+        default: launch_vector_L<VM, 32>(A, v, R, s); break;
     }
 }
 
@@ -676,10 +710,27 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
 static double row_mean(const Mat &A) { return A.n_rows > 0 ? (double)A.nnz / (double)A.n_rows : 0.0; }
 
 int crs_row_cut(const Mat &A) {
+    const double mean = row_mean(A);
     const int L = A.kopt.lanes;
     double cut = 16.0 * L;
-    if (L < 32) cut = std::max(cut, (L <= 4 ? 3 : 2) * row_mean(A));
+    if (L == 1) cut = mean >= 7 && mean <= 16 ? 2 * mean : A.kopt.rows_per_warp == 1 ? kShortRow : kShortRows;
+    else if (L < 32) cut = std::max(cut, (L <= 4 ? 3 : 2) * mean);
     return (int)std::min(cut, 1e9);
+}
+
+// One lane a row: four sets of rows a warp for the shortest rows, which are
+// bound by the loads in flight (one, two and four sets, us: 8M rows of one
+// entry, FP64 89, 58 and 44, FP32 93, 48 and 35; 4M rows of two, FP64 50, 33
+// and 33, FP32 50, 28 and 25), two for light tails in FP64 (crs_short_kernel),
+// one from five entries on, where heavy tails are as likely, and in FP32, which
+// pays more for the step out of line (rows of mean 2.5 with a log-normal
+// tail: 43 us with one set, 55 with two).
+int crs_default_rows(const Mat &A) {
+    const double mean = row_mean(A);
+    if (A.kopt.lanes > 1) return 4;
+    if (mean == 0) return 1;
+    if (A.dtype == GBSP_F64) return mean < 1.5 ? 4 : mean < 5 ? 2 : 1;
+    return mean < 2.25 ? 4 : 1;
 }
 
 void crs_default_opts(Mat &A) {
@@ -689,7 +740,7 @@ void crs_default_opts(Mat &A) {
                       : mean < (f64 ? 192 : 120) ? 16 : 32;
     A.kopt.kernel = GBSP_KERNEL_VECTOR;
     A.kopt.lanes = lanes;
-    A.kopt.rows_per_warp = lanes == 1 ? 1 : lanes == 4 && mean >= 24 ? 2 : 4;
+    A.kopt.rows_per_warp = lanes == 4 && mean >= 24 ? 2 : crs_default_rows(A);
     A.default_rows = A.kind == KIND_CRS;
     A.kopt.tile = 2048;
     A.kopt.rhs_tile = 16;

@@ -163,16 +163,23 @@ gbsp_status crs_dval_launch(const Mat &A, int32_t m, const void *G, int64_t g_ro
                             const void *X, int64_t x_row, int64_t x_t, void *dval, int32_t accumulate,
                             cudaStream_t s);
 void crs_default_opts(Mat &A);
-// VECTOR, more than one lane a row: rows longer than this are taken out of
-// their group's loop for the whole warp (in the batched product too, so that
-// both return the same bits).  The warp waits for its longest row, so a group
-// that is still at it after 16 steps gives it up: Zipf rows, 4 x 4: 516 us
-// with a limit of 512 entries, 356 us with 32 steps, 297 us with 16.  But not
-// a row like many others, hence three times the mean with few lanes (8M
-// entries, 70% of the rows of 9 and 30% of 71, 4 x 2: 65 us with 16 steps, 50
-// us) and twice with 8 and 16 (three times: 70% of the rows of 50 and 30% of
-// 382, 16 x 4: 38 -> 55 us); a whole warp a row has six loads a lane in flight
-// past 512 entries, but R in its loop.
+int crs_default_rows(const Mat &A);  // VECTOR rows a group for the handle's lanes
+// VECTOR: rows longer than this are taken out of their group's loop, with one
+// lane a row for eight lanes or the whole warp (rows.cuh), with more for the
+// whole warp (in the batched product too, so that both return the same bits).
+//   Several lanes: the warp waits for its longest row, so a group that is
+//   still at it after 16 steps gives it up: Zipf rows, 4 x 4: 516 us with a
+//   limit of 512 entries, 356 us with 32 steps, 297 us with 16.  But not a row
+//   like many others, hence three times the mean with few lanes (8M entries,
+//   70% of the rows of 9 and 30% of 71, 4 x 2: 65 us with 16 steps, 50 us) and
+//   twice with 8 and 16 (three times: 70% of the rows of 50 and 30% of 382,
+//   16 x 4: 38 -> 55 us); a whole warp a row has six loads a lane in flight
+//   past 512 entries, but R in its loop.
+//   One lane: 8, the most that heavy tails bear (Zipf rows, 4M: 8, 12 and 16:
+//   170, 178 and 183 us); 12 where several sets of rows a warp were chosen,
+//   for light tails (hybrid remainder, 5.0 a row, two sets: 8, 12 and 16: 146,
+//   125 and 125 us); and where one lane is asked for on rows of 7 to 16,
+//   twice the mean (13 a row: 57 us with 8, 30 us).
 int crs_row_cut(const Mat &A);
 
 // jds.cu ----------------------------------------------------------------

@@ -59,6 +59,7 @@ __device__ __forceinline__ int chunk_row(int32_t rs, int32_t re, int32_t cb, int
     }
     return r;
 }
+
 // Flagged rows with the whole warp on each row in turn.  Every lane passes
 // its group's mask (bit i: row first + i * step is long; only `leader`
 // lanes' masks are read); lanes stride through a row U loads deep, with the
@@ -88,7 +89,7 @@ __device__ __noinline__ void crs_warp_long_rows(bool leader, unsigned mask, int6
             const int s0 = __ldg(row_ptr + r), s1 = __ldg(row_ptr + r + 1);
             Acc<VM> a;
             a.init();
-                        int c[U];
+            int c[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) c[u] = s0 + lane + 32 * u < s1 ? __ldg(col + s0 + lane + 32 * u) : -1;
             auto entries = [&](auto N, int j) {  // N per lane from entry j + lane on
@@ -121,18 +122,47 @@ __device__ __noinline__ void crs_warp_long_rows(bool leader, unsigned mask, int6
     }
 }
 
-// VECTOR with one lane a row, R sets of 32 consecutive rows from `base` on:
-// rows of up to kShortRow entries by one lane, the loads of 8 / R slots of all
-// sets issued together; rows of up to kMidRow by eight lanes; longer ones by
-// the whole warp.  Without the two upper classes a warp runs to its longest
-// row: on the Zipf rows (5.5 entries a row, up to 5000) 1098 us against 168
-// us now (181 us with a fixed number of slots a step, see with_slots); what
-// is left there is FP64 issue (idle lanes issue too) and the latency of the
-// longest rows.  kMidRow 32, 64 and 128 gave 198, 185 and 183 us.  A row's arithmetic depends on its length alone,
-// so the batched product, which cuts the rows elsewhere, returns the same
-// bits.
-constexpr int kShortRow = 8;
+// VECTOR with one lane a row: rows of up to `cut` entries (crs_row_cut) by one
+// lane; rows of up to kMidRow by eight lanes; longer ones by the whole warp.
+// Without the two upper classes a warp runs to its longest row: on the Zipf
+// rows (5.5 entries a row, up to 5000) 1098 us against 168 us now (181 us with
+// a fixed number of slots a step, see with_slots); what is left there is FP64
+// issue (idle lanes issue too) and the latency of the longest rows.  kMidRow
+// 32, 64 and 128 gave 198, 185 and 183 us.  A row's arithmetic depends on its
+// length alone, so the batched product, which cuts the rows elsewhere,
+// returns the same bits.
 constexpr int kMidRow = 128;
+
+// The slots of R sets of 32 rows, one row a lane, to the longest: k0[i] and
+// n[i] the lane's row of set i (n < 1: none).  The loads of U slots of all
+// sets are issued together.
+template <int VM, int R, int U>
+__device__ __forceinline__ void lane_sums(Acc<VM> (&acc)[R], const int (&k0)[R], const int (&n)[R],
+                                          const int32_t *__restrict__ col,
+                                          const typename ValT<VM>::T *__restrict__ val,
+                                          const typename ValT<VM>::T *__restrict__ x, int64_t ldx, int longest) {
+    typedef typename ValT<VM>::T T;
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i].init();
+    for (int j = 0; j < longest; j += U)
+        with_slots<VM, U>(min(longest - j, U), [&](auto N) {
+            int c[R][N.value];
+            T v[R][N.value];
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int u = 0; u < N.value; ++u) {
+                    const bool ok = j + u < n[i];
+                    c[i][u] = ok ? __ldg(col + k0[i] + j + u) : -1;
+                    v[i][u] = ok ? __ldg(val + k0[i] + j + u) : T(0);
+                }
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int u = 0; u < N.value; ++u)
+                    if (c[i][u] >= 0) acc[i].add(v[i][u], ld_vec(x + (int64_t)c[i][u] * ldx));
+        });
+}
 
 // Rows base + i, i in the bits of `todo` (the same in every lane; lane i
 // passes the row's bounds s0, s1): eight lanes a row, four rows at a time.
@@ -182,66 +212,65 @@ __device__ __forceinline__ void crs_mid_rows(unsigned todo, int64_t base, int s0
     }
 }
 
-template <int VM, int R>
-__device__ __forceinline__ void crs_short_rows(int64_t base, int64_t n_rows, const int32_t *__restrict__ row_ptr,
+// 32 consecutive rows from `base` on, class by class, the loads of eight slots
+// of the short rows issued together.  CUT: the cut where it is a constant
+// (kShortRow), else 0: FP32 Zipf rows, 4M, 138 us against 148 us with the
+// cut in a register.
+constexpr int kShortRow = 8, kShortRows = 12;  // one set of rows a warp, several
+template <int VM, int CUT>
+__device__ __forceinline__ void crs_short_rows(int cut, int64_t base, int64_t n_rows,
+                                               const int32_t *__restrict__ row_ptr,
                                                const int32_t *__restrict__ col,
                                                const typename ValT<VM>::T *__restrict__ val,
                                                const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
                                                typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
     typedef typename ValT<VM>::T T;
-    constexpr int U = kShortRow / R;
-    const int lane = threadIdx.x & 31;
-    int k0[R], n[R];
-    int len = 0;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const int64_t r = base + 32 * i + lane;
-        k0[i] = 0;
-        n[i] = 0;
-        if (r < n_rows) {
-            k0[i] = __ldg(row_ptr + r);
-            n[i] = __ldg(row_ptr + r + 1) - k0[i];
-        }
-        if (n[i] <= kShortRow) len = max(len, n[i]);
+    constexpr int U = 8;
+    if (CUT > 0) cut = CUT;
+    const int64_t r = base + (threadIdx.x & 31);
+    int k0 = 0, n = 0, len = 0;
+    if (r < n_rows) {
+        k0 = __ldg(row_ptr + r);
+        n = __ldg(row_ptr + r + 1) - k0;
     }
-    Acc<VM> acc[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) acc[i].init();
+    if (n <= cut) len = n;
+    Acc<VM> acc;
+    acc.init();
     const int longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
     for (int j = 0; j < longest; j += U)
         with_slots<VM, U>(min(longest - j, U), [&](auto N) {
-            int c[R][N.value];
-            T v[R][N.value];
+            int c[N.value];
+            T v[N.value];
 #pragma unroll
-            for (int i = 0; i < R; ++i)
+            for (int u = 0; u < N.value; ++u) {
+                const bool ok = j + u < n && n <= cut;
+                c[u] = ok ? __ldg(col + k0 + j + u) : -1;
+                v[u] = ok ? __ldg(val + k0 + j + u) : T(0);
+            }
 #pragma unroll
-                for (int u = 0; u < N.value; ++u) {
-                    const bool ok = j + u < n[i] && n[i] <= kShortRow;
-                    c[i][u] = ok ? __ldg(col + k0[i] + j + u) : -1;
-                    v[i][u] = ok ? __ldg(val + k0[i] + j + u) : T(0);
-                }
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int u = 0; u < N.value; ++u)
-                    if (c[i][u] >= 0) acc[i].add(v[i][u], ld_vec(x + (int64_t)c[i][u] * ldx));
+            for (int u = 0; u < N.value; ++u)
+                if (c[u] >= 0) acc.add(v[u], ld_vec(x + (int64_t)c[u] * ldx));
         });
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const int64_t r = base + 32 * i + lane;
-        if (r < n_rows && n[i] <= kShortRow) {
-            if (accumulate) acc[i].add_value(y[r * ldy]);
-            y[r * ldy] = acc[i].result();
-        }
+    if (r < n_rows && n <= cut) {
+        if (accumulate) acc.add_value(y[r * ldy]);
+        y[r * ldy] = acc.result();
     }
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-        const unsigned mid = __ballot_sync(0xffffffffu, n[i] > kShortRow && n[i] <= kMidRow);
-        if (mid) crs_mid_rows<VM>(mid, base + 32 * i, k0[i], k0[i] + n[i], col, val, x, ldx, y, ldy, accumulate);
-        const unsigned big = __ballot_sync(0xffffffffu, n[i] > kMidRow);
-        if (big)
-            crs_warp_long_rows<VM, 4>(lane == 0, big, base + 32 * i, 1, row_ptr, col, val, x, ldx, y, ldy, accumulate);
-    }
+    const unsigned mid = __ballot_sync(0xffffffffu, n > cut && n <= kMidRow);
+    if (mid) crs_mid_rows<VM>(mid, base, k0, k0 + n, col, val, x, ldx, y, ldy, accumulate);
+    const unsigned big = __ballot_sync(0xffffffffu, n > cut && n > kMidRow);
+    if (big)
+        crs_warp_long_rows<VM, 4>((threadIdx.x & 31) == 0, big, base, 1, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+}
+
+// The 32-row sets of [base, end), out of line.
+template <int VM, int CUT>
+__device__ __noinline__ void short_rows_cut(int cut, int64_t base, int64_t end, const int32_t *__restrict__ row_ptr,
+                                            const int32_t *__restrict__ col,
+                                            const typename ValT<VM>::T *__restrict__ val,
+                                            const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
+                                            typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+    for (; base < end; base += 32)
+        crs_short_rows<VM, CUT>(cut, base, end, row_ptr, col, val, x, ldx, y, ldy, accumulate);
 }
 
 // SpMM: lanes per row of a pass over k right-hand sides, at most `tile` (16

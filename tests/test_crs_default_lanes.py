@@ -25,3 +25,10 @@ def shape(n_rows, nnz, dtype):
 def test_long_rows(mean, f64, f32):
     assert shape(64, 64 * mean, 0) == (f64, 4)
     assert shape(64, 64 * mean, 1) == (f32, 4)
+
+
+@pytest.mark.parametrize("nnz,f64,f32", [(0, 1, 1), (1, 4, 4), (149, 4, 4), (150, 2, 4), (224, 2, 4), (225, 2, 1),
+                                         (499, 2, 1), (500, 1, 1), (599, 1, 1)])
+def test_short_rows(nnz, f64, f32):
+    assert shape(100, nnz, 0) == (1, f64)
+    assert shape(100, nnz, 1) == (1, f32)

@@ -59,3 +59,31 @@ def _check(A, shapes, dtype):
 def test_cut_by_mean(base, factor, dtype):
     A = _matrix(2003 if base > 100 else 8003, base, factor)
     _check(A, [(l, r) for l in (2, 4, 8, 16, 32) for r in (1, 2, 4)], dtype)
+
+
+ONE_LANE = [(1, 1), (1, 2), (1, 4)]
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("n", [1, 31, 33, 64, 65, 127, 129, 20_011])
+@pytest.mark.parametrize("every", [1, 5, 200])
+def test_one_lane_short(n, every, dtype):
+    """Short rows with others around the one-lane limits (8 with one set of
+    rows a warp, 12 with several) and the warp's (128) in every position; steps
+    without any, too."""
+    lens = S.randint(3, 1, np.arange(n), 0, 4).astype(np.int64)
+    at = np.arange(every // 2, n, every)
+    lens[at] = np.resize([8, 9, 12, 13, 0, 128, 129, 300] if every > 1 else [0, 0, 1, 8, 9, 0, 12, 13, 2, 0, 4],
+                         at.size)
+    row_ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(lens, out=row_ptr[1:])
+    nnz = int(row_ptr[-1])
+    col = S.randint(7, 1, np.arange(nnz), 0, 50_020)
+    _check(S.CRS(n, 50_021, row_ptr.astype(np.int32), col.astype(np.int32), S.vector(nnz, 9)), ONE_LANE, dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("base", [6, 7, 13, 16, 17, 30])
+def test_one_lane_asked_for(base, dtype):
+    """One lane on longer rows: the limit is twice the mean from 7 to 16."""
+    _check(_matrix(4001, base, 2), ONE_LANE, dtype)
