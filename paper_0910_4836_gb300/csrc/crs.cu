@@ -398,18 +398,20 @@ crs_runs_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 constexpr int kRowCta = 64;  // see row_grid
 
 // SpMM: the lanes of a warp form 32 / W groups of W lanes, one lane per
-// right-hand side of the pass.  FP64: a warp takes about 16 rows and the
+// right-hand side of the pass.  FP64: a warp takes up to 16 rows and the
 // groups take them by length (spmm_rows): bound by FP64 issue (90% of it on
 // the HH-like matrix, N = 1,201,200: k = 16 487 -> 452 us, k = 5 281 -> 182
-// us, k = 3 158 -> 131 us).  Few rows a warp keep the rows that are in work at
-// one time close together: 32 instead of 16 took 540 us, X's rows leaving L2
-// before the other diagonals come back to them; fewer than 64 warps an SM
-// (more than 32 registers) cost as much as longer steps gain.  Where
-// the groups cover those rows in one round, and in FP32, which is not bound
-// by FP64 issue, a group takes one row in matrix order.
+// us, k = 3 158 -> 131 us; rows of one length only lose by it, 5% at 1.2M rows
+// of 27).  Few rows a warp keep the rows that are in work at one time close
+// together: 32 instead of 16 took 540 us, X's rows leaving L2 before the other
+// diagonals come back to them; fewer than 64 warps an SM (more than 32
+// registers) cost as much as longer steps gain.  Fewer rows still where 16
+// would not fill the GPU twice (launch_spmm).  Where the groups cover those
+// rows in one round, with one group a warp, which pairs nothing, and in FP32,
+// which is not bound by FP64 issue, a group takes one row in matrix order.
 template <int VM, int W>
 __host__ __device__ constexpr int spmm_rows_per_warp() {
-    return VM == VM_F64 && 32 / W < 16 ? 16 / (32 / W) * (32 / W) : 32 / W;
+    return VM == VM_F64 && 32 / W > 1 && 32 / W < 16 ? 16 / (32 / W) * (32 / W) : 32 / W;
 }
 
 template <int VM, int W>
@@ -417,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, spmm_rows_per_warp<VM, W>() > 32 / W
 crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                 const typename ValT<VM>::T *__restrict__ X, int64_t ldx,
-                typename ValT<VM>::T *__restrict__ Y, int64_t ldy, int k, int c0, int accumulate) {
+                typename ValT<VM>::T *__restrict__ Y, int64_t ldy, int k, int c0, int accumulate, int rw) {
     typedef typename ValT<VM>::T T;
     __shared__ uint8_t order[kRowCta / 32][32];
     constexpr int G = 32 / W, RW = spmm_rows_per_warp<VM, W>();
@@ -425,8 +427,8 @@ crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
     const bool active = grp < G && cc < k;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (RW > G) {
-        if (warp * RW < n_rows)
-            spmm_rows<VM, W>(warp * RW, (int)min((int64_t)RW, n_rows - warp * RW), active, order[threadIdx.x >> 5],
+        if (warp * rw < n_rows)
+            spmm_rows<VM, W>(warp * rw, (int)min((int64_t)rw, n_rows - warp * rw), active, order[threadIdx.x >> 5],
                              row_ptr, col, val, X + cc, ldx, Y + cc, ldy, accumulate);
         return;
     }
@@ -673,11 +675,17 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
     typedef typename ValT<VM>::T T;
     const int w = spmm_width(v.k, A.kopt.rhs_tile);
     with_spmm_width(w, [&](auto W) {
-        const int grid = row_grid(ceil_div(A.n_rows, (int64_t)spmm_rows_per_warp<VM, W.value>()));
+        constexpr int G = 32 / W.value, RW = spmm_rows_per_warp<VM, W.value>();
+        // at least two waves of 64 warps an SM (16 rows a warp everywhere, us,
+        // k = 16: 10,000 rows of U{1..33} 32 -> 13.5, 40,000 of 27 40 -> 36;
+        // one or four waves: 150,000 rows of U{1..33} 97 or 102 against 94)
+        const int64_t fill = A.n_rows / ((int64_t)num_sms() * 64 * 2);
+        const int rw = (int)std::max<int64_t>(G, std::min<int64_t>(RW, fill) / G * G);
+        const int grid = row_grid(ceil_div(A.n_rows, (int64_t)rw));
         for (int c0 = 0; c0 < v.k; c0 += W.value)
             crs_spmm_kernel<VM, W.value><<<grid, kRowCta, 0, s>>>(
                 A.n_rows, A.row_ptr, A.col, static_cast<const T *>(A.val), static_cast<const T *>(v.x), v.ldx,
-                static_cast<T *>(v.y), v.ldy, v.k, c0, v.accumulate);
+                static_cast<T *>(v.y), v.ldy, v.k, c0, v.accumulate, rw);
     });
 }
 
