@@ -368,7 +368,11 @@ __global__ void __launch_bounds__(256) jds_block_kernel(JdsArgs a) {
 // instruction count is what bounds the walk: N = 1.2M 48.4 -> 45.6 us, 3M
 // 108.2 -> 107.5, a 1000 x 1000 Laplacian 22.8 -> 18.5, FP32 compensated N =
 // 2M 59.5 -> 56.9; with vectors past L2's reach (6M), where HBM and the
-// gathers do, the plain last step is faster: 211.0 against 213.6 us.
+// gathers do, the plain last step is faster: 211.0 against 213.6 us.  Plain too
+// for eight right-hand sides a thread, where the second copy of the products
+// takes registers (58 for 52; k = 7: 130 against 110 us, 230,000 rows of
+// U{1..33}), and in FP64 with x gathered through the permutation, where the
+// exact step spills (2M rows of U{1..5}: 25.0 against 23.6 us).
 template <int VM, int U, int KT, bool PLAIN, bool EXACT>
 __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
     typedef typename ValT<VM>::T T;
@@ -479,7 +483,7 @@ __device__ __forceinline__ void sell_walk(const JdsArgs &a) {
 
 template <int VM, int U, int KT, bool PLAIN>
 __global__ void __launch_bounds__(1024) sell_kernel(JdsArgs a) {
-    sell_walk<VM, U, KT, PLAIN, true>(a);
+    sell_walk<VM, U, KT, PLAIN, KT != 8 && (VM != VM_F64 || KT > 1 || PLAIN)>(a);
 }
 
 // The plain one-vector FP64 walk compiled for two CTAs per SM: at the same
