@@ -223,6 +223,12 @@ __device__ __forceinline__ void jds_deep_items(const JdsArgs &a, int64_t n_items
     }
 }
 
+// The deep items alone, before the walk (launch_row says when).
+template <int VM>
+__global__ void __launch_bounds__(256) jds_deep_kernel(JdsArgs a, int64_t n_items) {
+    jds_deep_items<VM>(a, n_items, blockIdx.x, gridDim.x);
+}
+
 // A split walk in one launch: the first blocks take the deep items, which are
 // the longer chains, the others walk the rows.  Bound by the L1TEX stage of
 // the gathers; the walk's warps and the deep items' fill each other's waits.
@@ -718,7 +724,18 @@ static int row_grid(int64_t rows) {
 
 template <int VM, int U>
 static void launch_row(const JdsArgs &a, int R, cudaStream_t s, int64_t items = 0) {
-    if (items > 0) {
+    // Apart, one after the other, where the walk and the deep items fit one
+    // kernel badly and both fill the GPU.  U = 16: the walk's registers leave
+    // two CTAs an SM (4M Zipf rows, depth 2, chunk 8: joint 385, apart 295 us).
+    // U = 1 and 8: the joint kernel's occupancy is below the walk's own, which
+    // counts where many rows go deep (5M rows of U{1..29}, FP32, depth 16: 285
+    // and 223 against 240 and 209 us).
+    const bool apart = U >= 16 ? items >= (int64_t)num_sms() * 8
+                               : (U == 1 || (U == 8 && VM != VM_F64)) && items >= (int64_t)num_sms() * 32 && a.split_rows * 4 > a.n_rows;
+    if (items > 0 && apart) {
+        const unsigned db = (unsigned)std::min<int64_t>(items, (int64_t)num_sms() * 16);
+        jds_deep_kernel<VM><<<db, 256, 0, s>>>(a, items);
+    } else if (items > 0) {
         const unsigned g1 = (unsigned)limit_grid(row_grid(a.n_rows), a.grid_limit);
         const unsigned db = (unsigned)std::min<int64_t>(items, (int64_t)num_sms() * 16);
         if (!a.x_perm && a.ldx == 1) jds_split_kernel<VM, U, true><<<db + g1, 256, 0, s>>>(a, items, (int)db);

@@ -46,3 +46,27 @@ def test_split_walk_chunks(perm, dtype):
             Y2 = torch.zeros((n, 2), dtype=dtype, device="cuda")
             J.spmm(X2[:, 1:], out=Y2[:, :1], basis=1)
             assert np.array_equal(host(Y2[:, 0]), ref), (unroll, depth, chunk)
+
+
+@pytest.mark.parametrize("unroll", [1, 8, 16])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_split_apart(unroll, dtype):
+    """Deep items enough to fill the GPU, on rows most of which go deep: the
+    deep items are launched before the walk.  Integer data, any order exact."""
+    n = 60_000
+    lens = S.randint(3, 1, np.arange(n), 0, 50).astype(np.int64)
+    row_ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(lens, out=row_ptr[1:])
+    nnz = int(row_ptr[-1])
+    A = S.integer_values(S.CRS(n, n, row_ptr.astype(np.int32), S.randint(7, 1, np.arange(nnz), 0, n - 1).astype(
+        np.int32), S.vector(nnz, 9)), 4, 8)
+    x, y0 = S.int_vector(n, 5, 16), S.int_vector(n, 6, 100)
+    ref = O.crs_spmv(A, x)
+    J = crs(A, dtype).to_jds("NUJDS", "symmetric", unroll=unroll)
+    for depth, chunk in ((1, 1), (9, 1), (49, 8)):
+        J.split(depth, chunk)
+        for limit in (0, 3):
+            J.set_grid_limit(limit)
+            assert np.array_equal(host(J.spmv_original(dev(x, dtype))), ref), (depth, chunk, limit)
+            y = J.spmv(J.permute(dev(x, dtype)), out=J.permute(dev(y0, dtype)), accumulate=True)
+            assert np.array_equal(host(J.permute(y, back=True)), ref + y0), (depth, chunk, limit)
