@@ -215,7 +215,7 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
 template <int KTMAX>
 __device__ __forceinline__ int clamp_tile(int kt) { return kt < KTMAX ? kt : KTMAX; }
 
-template <int VM, int KTMAX, bool CRS1>
+template <int VM, int KTMAX, bool CRS1, bool CRSK>
 __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*order)[32]) {
     if (m.kind == KIND_JDS && m.format == GBSP_SELL) {
         int KT = 1;
@@ -246,7 +246,7 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*
                 case 16: batch_crs_rows<VM, 16>(m, rb, re); break;
                 default: batch_crs_rows<VM, 32>(m, rb, re); break;
             }
-        } else {
+        } else if constexpr (CRSK) {
             with_spmm_width(spmm_width(m.k, m.rhs_tile), [&](auto W) {
                 for (int c0 = 0; c0 < m.k; c0 += W.value) batch_crs_spmm_rows<VM, W.value>(m, rb, re, c0, order);
             });
@@ -273,9 +273,11 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*
 // issue and by the latency of its gathers, and 32 registers with some spills
 // beat five or six CTAs with none (256 matrices, mixed k, FP64: 1736, 1666
 // and 1603 us for five, six and eight; one kernel with 64 registers for any
-// k > 4 took 2160 us).
-template <int KTMAX, bool CRS1>
-__global__ void __launch_bounds__(kBatchThreads, KTMAX > 1 ? 4 : CRS1 ? 5 : 8)
+// k > 4 took 2160 us).  With one on CRS items five (64 matrices, k = 1 and 16 in
+// turn: 791 us, 893 with four), but four without FP64 items (FP32: 902 us with
+// five, 671 with four).
+template <int KTMAX, bool CRS1, bool CRSK, bool F64>
+__global__ void __launch_bounds__(kBatchThreads, KTMAX > 1 || !F64 ? 4 : CRS1 ? 5 : 8)
 batch_kernel(const BatchMat *__restrict__ mats, const BatchWork *__restrict__ work, int64_t n_work,
              int32_t *counter, const volatile int32_t *ready, int32_t *status) {
     __shared__ int64_t next[2];
@@ -311,9 +313,13 @@ batch_kernel(const BatchMat *__restrict__ mats, const BatchWork *__restrict__ wo
         if (w >= n_work) break;
         const BatchWork wk = work[w];
         const BatchMat m = mats[wk.mat];
-        if (m.vm == VM_F64) batch_item<VM_F64, KTMAX, CRS1>(m, wk.rb, wk.re, order);
-        else if (m.vm == VM_F32C) batch_item<VM_F32C, KTMAX, CRS1>(m, wk.rb, wk.re, order);
-        else batch_item<VM_F32, KTMAX, CRS1>(m, wk.rb, wk.re, order);
+        if (m.vm == VM_F64) {
+            if constexpr (F64) batch_item<VM_F64, KTMAX, CRS1, CRSK>(m, wk.rb, wk.re, order);
+        } else if (m.vm == VM_F32C) {
+            batch_item<VM_F32C, KTMAX, CRS1, CRSK>(m, wk.rb, wk.re, order);
+        } else {
+            batch_item<VM_F32, KTMAX, CRS1, CRSK>(m, wk.rb, wk.re, order);
+        }
         if (threadIdx.x == 0) next[i ^ 1] = atomicAdd(counter, 1);
         // every thread has read next[i]; next[i ^ 1] is written and visible
         __syncthreads();
@@ -338,13 +344,18 @@ struct gbsp_batch_s {
 namespace {
 
 // The kernel instance decides the registers, hence the CTAs per SM: the
-// widest tile of JDS-family items with several right-hand sides, and
-// whether any CRS item has one (CRS items with several need neither).
-const void *batch_instance(int kmax, bool crs1) {
-    if (kmax > 4) return reinterpret_cast<const void *>(batch_kernel<8, true>);
-    if (kmax > 1) return reinterpret_cast<const void *>(batch_kernel<4, true>);
-    if (crs1) return reinterpret_cast<const void *>(batch_kernel<1, true>);
-    return reinterpret_cast<const void *>(batch_kernel<1, false>);
+// widest tile of JDS-family items with several right-hand sides (kmax),
+// whether any CRS item has one (crs1; CRS items with several, crsk, need
+// neither), and whether there are FP64 items.  Without CRS or FP64 items four
+// right-hand sides do better in a kernel that has no code for them (64 JDS
+// matrices, FP32: 490 -> 442 us; FP64: 512 -> 572).
+const void *batch_instance(int kmax, bool crs1, bool crsk, bool f64) {
+    if (kmax > 4) return reinterpret_cast<const void *>(batch_kernel<8, true, true, true>);
+    if (kmax > 1 && !crs1 && !crsk && !f64) return reinterpret_cast<const void *>(batch_kernel<4, false, false, false>);
+    if (kmax > 1) return reinterpret_cast<const void *>(batch_kernel<4, true, true, true>);
+    if (crs1 && crsk && !f64) return reinterpret_cast<const void *>(batch_kernel<1, true, true, false>);
+    if (crs1) return reinterpret_cast<const void *>(batch_kernel<1, true, true, true>);
+    return reinterpret_cast<const void *>(batch_kernel<1, false, true, true>);
 }
 
 constexpr int64_t kCounterBytes = 256;
@@ -510,12 +521,13 @@ gbsp_status gbsp_batch_create(int32_t n, const gbsp_batch_item *items, int32_t c
                                   cudaMemcpyHostToDevice, s));
     GBSP_CUDA(cudaStreamSynchronize(s));  // host vectors go out of scope
     int kmax = 1;
-    bool crs1 = false;
+    bool crs1 = false, crsk = false, f64 = false;
     for (int32_t i = 0; i < n; ++i) {
         if (items[i].A->kind != KIND_CRS) kmax = std::max(kmax, (int)items[i].k);
-        else if (items[i].k == 1) crs1 = true;
+        else (items[i].k == 1 ? crs1 : crsk) = true;
+        f64 |= items[i].A->dtype == GBSP_F64;
     }
-    b->kernel = batch_instance(kmax, crs1);
+    b->kernel = batch_instance(kmax, crs1, crsk, f64);
     int per_sm = 0;
     GBSP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kBatchThreads, 0));
     b->grid = (int)std::max<int64_t>(1, std::min<int64_t>(b->n_work, (int64_t)num_sms() * std::max(per_sm, 1)));
