@@ -1247,16 +1247,16 @@ gather_values_kernel(int64_t nnz, const int32_t *__restrict__ tmap,
 // row, are read together and each source sector is fetched once; in entry
 // order the lanes of a warp would take one 8-byte value from each of 32
 // sectors and come back for the rest of those sectors a diagonal later.
-// Four slots' loads in flight: 27-point stencil 145 -> 110 us (JDS), 154 ->
-// 113 us (SELL).
+// U slots' loads in flight, four: 27-point stencil 145 -> 110 us (JDS), 154 ->
+// 113 us (SELL); one below 1.5 entries a row, where the other three are mostly
+// past the row: 2M rows of one entry 12.5 -> 8.9 us (JDS), 12.6 -> 10.7 us (SELL).
 // JDS storage (JDS, NBJDS, NUJDS): thread r walks the diagonals of permuted row r.
-template <typename T>
+template <typename T, int U>
 __global__ void jds_rows_gather_kernel(int64_t n, int64_t n_diag, const int32_t *__restrict__ jd_ptr,
                                        const int32_t *__restrict__ map, const T *__restrict__ src,
                                        T *__restrict__ dst) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    constexpr int U = 4;  // diagonals whose loads are in flight together
     for (int64_t d = 0; d < n_diag; d += U) {
         int32_t pos[U], k[U];
         T v[U];
@@ -1278,7 +1278,7 @@ __global__ void jds_rows_gather_kernel(int64_t n, int64_t n_diag, const int32_t 
 }
 
 // SELL: one warp per 32-row block, lane = row, slots as in the SELL walk.
-template <typename T>
+template <typename T, int U>
 __global__ void sell_rows_gather_kernel(int64_t n, int64_t nb, const int32_t *__restrict__ rlen,
                                         const int32_t *__restrict__ blk_ptr, const int32_t *__restrict__ map,
                                         const T *__restrict__ src, T *__restrict__ dst) {
@@ -1289,7 +1289,6 @@ __global__ void sell_rows_gather_kernel(int64_t n, int64_t nb, const int32_t *__
     const int32_t len = r < n ? __ldg(rlen + r) : 0;
     int64_t off = __ldg(blk_ptr + b);
     const int32_t width = __shfl_sync(0xffffffffu, len, 0);
-    constexpr int U = 4;  // slots whose loads are in flight together
     for (int32_t d = 0; d < width; d += U) {
         int64_t pos[U];
         int32_t k[U];
@@ -1309,34 +1308,30 @@ __global__ void sell_rows_gather_kernel(int64_t n, int64_t nb, const int32_t *__
     }
 }
 
+template <typename T, int U>
+static gbsp_status rows_gather(const Mat &J, bool jds_storage, const void *src, cudaStream_t s) {
+    T *dst = static_cast<T *>(const_cast<void *>(J.val));
+    const unsigned g = (unsigned)ceil_div(ceil_div(J.n_rows, 32) * 32, 256);
+    if (jds_storage)
+        jds_rows_gather_kernel<T, U><<<g, 256, 0, s>>>(J.n_rows, J.n_diag, J.jd_ptr, J.vmap,
+                                                       static_cast<const T *>(src), dst);
+    else
+        sell_rows_gather_kernel<T, U><<<g, 256, 0, s>>>(J.n_rows, ceil_div(J.n_rows, 32), J.rlen, J.blk_ptr, J.vmap,
+                                                        static_cast<const T *>(src), dst);
+    GBSP_LAUNCH_CHECK("value re-gather by rows");
+    return GBSP_OK;
+}
+
 gbsp_status jds_values_launch(const Mat &J, const void *src, cudaStream_t s) {
     if (J.nnz == 0) return GBSP_OK;
     const bool jds_storage = J.jd_ptr && (J.format == GBSP_JDS || J.format == GBSP_NBJDS ||
                                           J.format == GBSP_NUJDS || J.format == GBSP_JDS_LITERAL);
-    const bool f64 = J.dtype == GBSP_F64;
     void *dst = const_cast<void *>(J.val);
-    if (jds_storage) {
-        const unsigned g = (unsigned)ceil_div(J.n_rows, 256);
-        if (f64)
-            jds_rows_gather_kernel<double><<<g, 256, 0, s>>>(J.n_rows, J.n_diag, J.jd_ptr, J.vmap,
-                                                             static_cast<const double *>(src), static_cast<double *>(dst));
-        else
-            jds_rows_gather_kernel<float><<<g, 256, 0, s>>>(J.n_rows, J.n_diag, J.jd_ptr, J.vmap,
-                                                            static_cast<const float *>(src), static_cast<float *>(dst));
-        GBSP_LAUNCH_CHECK("jds_rows_gather_kernel");
-        return GBSP_OK;
-    }
-    if (J.format == GBSP_SELL && J.rlen && J.blk_ptr) {
-        const int64_t nb = ceil_div(J.n_rows, 32);
-        const unsigned g = (unsigned)ceil_div(nb * 32, 256);
-        if (f64)
-            sell_rows_gather_kernel<double><<<g, 256, 0, s>>>(J.n_rows, nb, J.rlen, J.blk_ptr, J.vmap,
-                                                              static_cast<const double *>(src), static_cast<double *>(dst));
-        else
-            sell_rows_gather_kernel<float><<<g, 256, 0, s>>>(J.n_rows, nb, J.rlen, J.blk_ptr, J.vmap,
-                                                             static_cast<const float *>(src), static_cast<float *>(dst));
-        GBSP_LAUNCH_CHECK("sell_rows_gather_kernel");
-        return GBSP_OK;
+    if (jds_storage || (J.format == GBSP_SELL && J.rlen && J.blk_ptr)) {
+        const bool one = 2 * J.nnz < 3 * J.n_rows;
+        if (J.dtype == GBSP_F64)
+            return one ? rows_gather<double, 1>(J, jds_storage, src, s) : rows_gather<double, 4>(J, jds_storage, src, s);
+        return one ? rows_gather<float, 1>(J, jds_storage, src, s) : rows_gather<float, 4>(J, jds_storage, src, s);
     }
     return gather_values_launch(J.nnz, J.vmap, src, dst, J.dtype, s);
 }
