@@ -348,11 +348,14 @@ gbsp_status gbsp_sell_stage(gbsp_handle sell, int32_t pages_per_group, int32_t m
  * adds the row's partial sums (deterministic; the grouping of the sum
  * differs from the unsplit walk): rows with at most 8 chunks add them in
  * chunk order, longer rows in a fixed lane-strided tree.  Two launches per
- * product, both on `stream` (capturable in a CUDA graph): one whose first
- * blocks sum the deep chunks while the others walk the rows, then the merge.
+ * product, all on `stream` (capturable in a CUDA graph): one whose first
+ * blocks sum the deep chunks while the others walk the rows, one row a thread
+ * whatever rows_per_warp says and gbsp_set_grid_limit bounding the walk's
+ * blocks alone, then the merge; three where chunks and rows each fill the GPU
+ * and would hinder each other in one launch (unroll 16; unroll 1 or, in FP32,
+ * 8 with more than a quarter of the rows deep).
  * Calls on one split handle must not overlap (they share the workspace).
- * k = 1 only (SpMM ignores the split).  depth = 0 removes the
- * split.
+ * k = 1 only (SpMM ignores the split).  depth = 0 removes the split.
  * Workspace bytes from gbsp_jds_split_bytes; 256-byte aligned; borrowed
  * until destroy or the next gbsp_jds_split.  Synchronises `stream`. */
 gbsp_status gbsp_jds_split_bytes(gbsp_handle jds, int32_t depth, int32_t chunk, int64_t *bytes);
@@ -750,7 +753,7 @@ gbsp_status gbsp_warp_sectors(gbsp_handle A, int32_t lanes, int32_t elem_bytes, 
  * Time the candidate kernels for `A` with k right-hand sides on the device
  * (CUDA events on `stream`, a few repetitions each, X and Y are scratch
  * vectors of the right sizes) and keep the fastest option set on the handle.
- * For CRS handles the candidates are VECTOR with lanes 2..32 and every
+ * For CRS handles the candidates are VECTOR with lanes 1..32 and every
  * rows_per_warp, RUNS in six shapes, and TILED (when prepared); for
  * JDS-family handles the formats sharing
  * the handle's storage and their block/unroll values.  *best receives the

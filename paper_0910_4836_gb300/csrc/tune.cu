@@ -21,14 +21,15 @@ struct Cand {
     int format, block, unroll;
 };
 
-typedef std::tuple<int, int, int64_t, int64_t, int64_t, int, int, int, int, int> TuneKey;
+typedef std::tuple<int, int, int64_t, int64_t, int64_t, int, int, int, int, int, int, int> TuneKey;
 
 static std::mutex g_tune_mu;
 static std::map<TuneKey, std::pair<Cand, float>> g_tune_cache;
 
 static TuneKey key_of(const Mat &A, int k) {
     return TuneKey(A.kind, A.kind == KIND_JDS ? (A.built_block > 0 ? A.format : -1) : -1, A.n_rows, A.n_cols,
-                   A.nnz, k, A.dtype, A.kopt.accum, A.tile_rows != nullptr ? A.tile : 0, A.device);
+                   A.nnz, k, A.dtype, A.kopt.accum, A.tile_rows != nullptr ? A.tile : 0, A.device,
+                   A.split_k > 0 ? A.split_depth : 0, A.split_k > 0 ? A.split_chunk : 0);
 }
 
 static void apply(Mat &A, const Cand &c) {
@@ -73,7 +74,7 @@ static std::vector<Cand> candidates(const Mat &A, int k) {
     base.unroll = A.unroll;
     if (A.kind == KIND_CRS) {
         if (k == 1) {
-            for (int l : {2, 4, 8, 16, 32})
+            for (int l : {1, 2, 4, 8, 16, 32})
                 for (int r : {1, 2, 4}) {
                     Cand c = base;
                     c.k.kernel = GBSP_KERNEL_VECTOR;
@@ -127,6 +128,7 @@ static std::vector<Cand> candidates(const Mat &A, int k) {
             for (int u : {2, 4, 8})
                 for (int r : {1, 2, 4}) {
                     if (u == 8 && r == 4) continue;
+                    if (r > 1 && A.split_k > 0) continue;  // a split walk takes one row a thread
                     c = base;
                     c.format = GBSP_NUJDS;
                     c.unroll = u;
