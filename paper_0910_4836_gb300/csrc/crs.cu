@@ -482,9 +482,15 @@ crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 //     = 2 .. 6 the steps' loads are issued together.  27-point stencil
 //     against the loop over m: m = 2 176 -> 128 us, m = 5 247 -> 239, m = 6 346 ->
 //     285 (FP64 issue alone takes 86, 215 and 258); FP32 m = 5 181 -> 136.
-//     Four at a time for more steps gained nothing (m = 8 387 against 375 us).  With the loop, several chunks in flight took
-//     72 registers and ran slower (m = 5: 287 us against 249 us); so did the
-//     shuffle-free row lookup with one or two chunks in flight (294-490 us).
+//     From seven steps on FP64 issue hides the loop's latency (m = 7 and 8 as
+//     instances 2% faster; FP32 would gain there still: 400,000 rows of 27,
+//     m = 7, 80 against 54 us); four steps at a time gained nothing (m = 8 387
+//     against 375 us).  Registers for four CTAs an SM: without the hint the
+//     loads do not all stay in flight (Zipf rows, 1M, m = 5 and 6: 228 and 256
+//     us, 250 and 297 without; six CTAs are no faster).  With the loop,
+//     several chunks in flight took 72 registers and ran slower (m = 5: 287 us
+//     against 249 us); so did the shuffle-free row lookup with one or two
+//     chunks in flight (294-490 us).
 constexpr int kDvalWarps = kThreads / 32;
 constexpr int kDvalU = 4;
 
@@ -530,7 +536,7 @@ crs_dval_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 }
 
 template <typename T, int M>
-__global__ void __launch_bounds__(kThreads, M == 0 ? 0 : M == 2 || M == 6 ? 6 : 4)
+__global__ void __launch_bounds__(kThreads, M == 0 ? 0 : 4)
 crs_dval_multi_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, int m, const T *__restrict__ G, int64_t g_row,
                 int64_t g_t, const T *__restrict__ X, int64_t x_row, int64_t x_t, T *__restrict__ dval,
