@@ -209,9 +209,8 @@ __device__ void batch_sell_rows(const BatchMat &m, int64_t rb, int64_t re, int c
 // tile the kernel instance carries (a batch without several right-hand sides
 // on such items runs an instance without the wide-tile code and its
 // registers; k = 16 runs as two 8-wide tiles at twice the occupancy of a
-// 16-wide one).  The tile width never
-// changes a result: every right-hand side is summed on its own, in the same
-// entry order.
+// 16-wide one).  The tile width never changes a result: every right-hand side
+// is summed on its own, in the same entry order.
 template <int KTMAX>
 __device__ __forceinline__ int clamp_tile(int kt) { return kt < KTMAX ? kt : KTMAX; }
 
@@ -232,7 +231,6 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*
             if constexpr (KTMAX >= 2) if (KT == 2) batch_sell_rows<VM, 2, false>(m, rb, re, c0);
             if constexpr (KTMAX >= 4) if (KT == 4) batch_sell_rows<VM, 4, false>(m, rb, re, c0);
             if constexpr (KTMAX >= 8) if (KT == 8) batch_sell_rows<VM, 8, false>(m, rb, re, c0);
-            if constexpr (KTMAX >= 16) if (KT >= 16) batch_sell_rows<VM, 16, false>(m, rb, re, c0);
         }
         return;
     }
@@ -262,7 +260,6 @@ __device__ void batch_item(const BatchMat &m, int64_t rb, int64_t re, uint8_t (*
                 if (KT == 2) batch_jds_rows<VM, 2>(m, rb, re, c0);
                 if constexpr (KTMAX >= 4) if (KT == 4) batch_jds_rows<VM, 4>(m, rb, re, c0);
                 if constexpr (KTMAX >= 8) if (KT == 8) batch_jds_rows<VM, 8>(m, rb, re, c0);
-                if constexpr (KTMAX >= 16) if (KT >= 16) batch_jds_rows<VM, 16>(m, rb, re, c0);
             }
         }
     }

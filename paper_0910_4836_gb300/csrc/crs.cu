@@ -497,9 +497,8 @@ constexpr int kDvalU = 4;
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 crs_dval_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
-                const int32_t *__restrict__ col, int m, const T *__restrict__ G, int64_t g_row,
-                int64_t g_t, const T *__restrict__ X, int64_t x_row, int64_t x_t, T *__restrict__ dval,
-                int accumulate) {
+                const int32_t *__restrict__ col, const T *__restrict__ G, int64_t g_row,
+                const T *__restrict__ X, int64_t x_row, T *__restrict__ dval, int accumulate) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarp = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -803,9 +802,9 @@ static void launch_dval(const Mat &A, int32_t m, const void *G, int64_t g_row, i
                         cudaStream_t s) {
     const int grid = grid_for(ceil_div(A.n_rows, 32));
     if (m == 1)
-        crs_dval_kernel<T><<<grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, m, static_cast<const T *>(G), g_row,
-                                                     g_t, static_cast<const T *>(X), x_row, x_t,
-                                                     static_cast<T *>(dval), accumulate);
+        crs_dval_kernel<T><<<grid, kThreads, 0, s>>>(A.n_rows, A.row_ptr, A.col, static_cast<const T *>(G), g_row,
+                                                     static_cast<const T *>(X), x_row, static_cast<T *>(dval),
+                                                     accumulate);
     else {
         auto go = [&](auto M) {
             crs_dval_multi_kernel<T, M.value><<<grid, kThreads, 0, s>>>(
