@@ -109,15 +109,17 @@ __device__ __forceinline__ void vector_sums(Acc<VM> (&acc)[R], const int (&k0)[R
 // rows are left out of the groups' loops and summed afterwards by the whole
 // warp.  Out of line, so that the common step keeps its registers and code
 // (with the cut in the common step the 4 x 4 shape took 76 us instead of 65 us
-// on the HH-like matrix of N = 1,201,200).
+// on the HH-like matrix of N = 1,201,200).  flags: the cut, negative to
+// accumulate: one argument more, of its own for the cut, cost the common step
+// registers too (27-point stencil, 4 x 2: 70.5 us against 68.6).
 template <int VM, int L, int R>
-__device__ __noinline__ void vector_step_cut(int cut, int64_t first, int64_t n_rows,
-                                             const int32_t *__restrict__ row_ptr,
+__device__ __noinline__ void vector_step_cut(int64_t first, int64_t n_rows, const int32_t *__restrict__ row_ptr,
                                              const int32_t *__restrict__ col,
                                              const typename ValT<VM>::T *__restrict__ val,
                                              const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
-                                             typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+                                             typename ValT<VM>::T *__restrict__ y, int64_t ldy, int flags) {
     constexpr int G = 32 / L;
+    const int cut = abs(flags), accumulate = flags < 0;
     int k0[R], k1[R];
     int len = 0;
     unsigned lmask = 0;
@@ -148,10 +150,10 @@ __device__ __noinline__ void vector_step_cut(int cut, int64_t first, int64_t n_r
 // call to the long-row step raised some shapes to 60.
 template <int VM, int L, int R>
 __global__ void __launch_bounds__(kThreads, R == 4 ? 5 : 6)
-crs_vector_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
+crs_vector_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                   const int32_t *__restrict__ col, const typename ValT<VM>::T *__restrict__ val,
                   const typename ValT<VM>::T *__restrict__ x, int64_t ldx,
-                  typename ValT<VM>::T *__restrict__ y, int64_t ldy, int accumulate) {
+                  typename ValT<VM>::T *__restrict__ y, int64_t ldy, int flags) {
     constexpr int G = 32 / L;
     constexpr int RW = G * R;
     const int grp = (threadIdx.x & 31) / L;
@@ -171,17 +173,17 @@ crs_vector_kernel(int cut, int64_t n_rows, const int32_t *__restrict__ row_ptr,
             }
             len = max(len, k1[i] - k0[i]);
         }
-        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)cut) {
+        if (__reduce_max_sync(0xffffffffu, (unsigned)len) > (unsigned)abs(flags)) {
             if constexpr (L == 1)
-                short_rows_cut<VM, kShortRows>(cut, base, min(base + RW, n_rows), row_ptr, col, val, x, ldx, y, ldy,
-                                               accumulate);
+                short_rows_cut<VM, kShortRows>(kShortRows, base, min(base + RW, n_rows), row_ptr, col, val, x, ldx, y, ldy,
+                                               flags < 0);
             else
-                vector_step_cut<VM, L, R>(cut, base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, accumulate);
+                vector_step_cut<VM, L, R>(base + grp, n_rows, row_ptr, col, val, x, ldx, y, ldy, flags);
             continue;
         }
         Acc<VM> acc[R];
         vector_sums<VM, L, R>(acc, k0, k1, len, col, val, x, ldx);
-        scatter_store<VM, L, R>(acc, base + grp, G, 0u, n_rows, y, ldy, accumulate);
+        scatter_store<VM, L, R>(acc, base + grp, G, 0u, n_rows, y, ldy, flags < 0);
     }
 }
 
@@ -613,9 +615,9 @@ template <int VM, int L, int R>
 static void launch_vector_R(const Mat &A, const VecArgs &v, cudaStream_t s) {
     typedef typename ValT<VM>::T T;
     const int grid = (int)limit_grid(row_grid(ceil_div(A.n_rows, (32 / L) * R)), A.grid_limit);
-    crs_vector_kernel<VM, L, R><<<grid, kRowCta, 0, s>>>(crs_row_cut(A), A.n_rows, A.row_ptr, A.col,
-                                                         static_cast<const T *>(A.val), static_cast<const T *>(v.x),
-                                                         v.ldx, static_cast<T *>(v.y), v.ldy, v.accumulate);
+    crs_vector_kernel<VM, L, R><<<grid, kRowCta, 0, s>>>(A.n_rows, A.row_ptr, A.col, static_cast<const T *>(A.val),
+                                                         static_cast<const T *>(v.x), v.ldx, static_cast<T *>(v.y),
+                                                         v.ldy, v.accumulate ? -crs_row_cut(A) : crs_row_cut(A));
 }
 
 template <int VM, int L>
