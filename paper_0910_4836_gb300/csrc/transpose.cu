@@ -462,9 +462,12 @@ static SplitPlan split_plan(const Mat &A) {
 }
 
 // Every column must fall into one of at most 2048 buckets of 8192 columns,
-// and a record's key into 64 bits.
+// and a record's key into 64 bits.  Columns of 2^20 entries in the mean are
+// too few buckets for the GPU, and a bucket is one CTA's, round after round:
+// 8M entries in 1, 3 and 30 columns, split / radix sort: 27.9 / 5.3, 9.6 / 2.4
+// and 1.2 / 1.8 ms.
 bool transpose_split_fits(const Mat &A) {
-    if (A.nnz <= 0 || A.n_cols > (int64_t)kMaxBuckets * kMaxWidth) return false;
+    if (A.nnz <= 0 || A.n_cols > (int64_t)kMaxBuckets * kMaxWidth || A.nnz >> 20 >= A.n_cols) return false;
     const SplitPlan p = split_plan(A);
     return p.bits.c + p.bits.e + bits_for((uint64_t)A.n_rows - 1) <= 64;
 }

@@ -50,6 +50,16 @@ def test_long_rows(name, columns):
     _check(lens.size, columns, lens, lambda k: S.randint(7, 1, np.arange(k), 0, columns - 1), torch.float64)
 
 
+@pytest.mark.parametrize("nnz", [(1 << 20) - 1, 1 << 20, 2_500_001])
+@pytest.mark.parametrize("columns", [1, 2])
+def test_few_columns(columns, nnz):
+    """2^20 entries a column and more go to the radix sort."""
+    lens = np.resize([7, 0, 3, 11], nnz // 5)
+    lens = lens[np.cumsum(lens) <= nnz]
+    lens = np.append(lens, nnz - lens.sum())
+    _check(lens.size, columns, lens, lambda k: S.randint(7, 1, np.arange(k), 0, columns - 1), torch.float64)
+
+
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 @pytest.mark.parametrize("longest", [47, 49, 64, 97, 127, 128, 129, 160, 300])
 def test_column_lengths(longest, dtype):
