@@ -489,7 +489,8 @@ crs_spmm_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 //     m = 7, 80 against 54 us); four steps at a time gained nothing (m = 8 387
 //     against 375 us).  Registers for four CTAs an SM: without the hint the
 //     loads do not all stay in flight (Zipf rows, 1M, m = 5 and 6: 228 and 256
-//     us, 250 and 297 without; six CTAs are no faster).  With the loop,
+//     us, 250 and 297 without; six CTAs are no faster, but for m = 2 with
+//     accumulation in FP64: 400,000 rows of 27, 64 against 76 us).  With the loop,
 //     several chunks in flight took 72 registers and ran slower (m = 5: 287 us
 //     against 249 us); so did the shuffle-free row lookup with one or two
 //     chunks in flight (294-490 us).
@@ -537,7 +538,7 @@ crs_dval_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
 }
 
 template <typename T, int M>
-__global__ void __launch_bounds__(kThreads, M == 0 ? 0 : 4)
+__global__ void __launch_bounds__(kThreads, M == 0 ? 0 : M == 2 ? 6 : 4)
 crs_dval_multi_kernel(int64_t n_rows, const int32_t *__restrict__ row_ptr,
                 const int32_t *__restrict__ col, int m, const T *__restrict__ G, int64_t g_row,
                 int64_t g_t, const T *__restrict__ X, int64_t x_row, int64_t x_t, T *__restrict__ dval,
