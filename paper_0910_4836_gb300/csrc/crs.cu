@@ -684,10 +684,13 @@ static void launch_spmm(const Mat &A, const VecArgs &v, cudaStream_t s) {
     const int w = spmm_width(v.k, A.kopt.rhs_tile);
     with_spmm_width(w, [&](auto W) {
         constexpr int G = 32 / W.value, RW = spmm_rows_per_warp<VM, W.value>();
-        // at least two waves of 64 warps an SM (16 rows a warp everywhere, us,
+        // At least two waves of 64 warps an SM (16 rows a warp everywhere, us,
         // k = 16: 10,000 rows of U{1..33} 32 -> 13.5, 40,000 of 27 40 -> 36;
-        // one or four waves: 150,000 rows of U{1..33} 97 or 102 against 94)
-        const int64_t fill = A.n_rows / ((int64_t)num_sms() * 64 * 2);
+        // one or four waves: 150,000 rows of U{1..33} 97 or 102 against 94);
+        // fewer with more groups, which take fewer rounds and of whose rows
+        // more are paired (k = 4, 230,000 rows of U{1..33}: 56 with two waves, 48.5)
+        const int64_t quarters = G <= 3 ? 8 : G == 4 ? 2 : 1;
+        const int64_t fill = 4 * A.n_rows / ((int64_t)num_sms() * 64 * quarters);
         const int rw = (int)std::max<int64_t>(G, std::min<int64_t>(RW, fill) / G * G);
         const int grid = row_grid(ceil_div(A.n_rows, (int64_t)rw));
         for (int c0 = 0; c0 < v.k; c0 += W.value)
