@@ -723,15 +723,16 @@ static int row_grid(int64_t rows) {
 }
 
 template <int VM, int U>
-static void launch_row(const JdsArgs &a, int R, cudaStream_t s, int64_t items = 0) {
+static void launch_row(const JdsArgs &a, int R, cudaStream_t s, int64_t items, bool mostly_shallow) {
     // Apart, one after the other, where the walk and the deep items fit one
     // kernel badly and both fill the GPU.  U = 16: the walk's registers leave
     // two CTAs an SM (4M Zipf rows, depth 2, chunk 8: joint 385, apart 295 us).
-    // U = 1 and 8: the joint kernel's occupancy is below the walk's own, which
-    // counts where many rows go deep (5M rows of U{1..29}, FP32, depth 16: 285
-    // and 223 against 240 and 209 us).
-    const bool apart = U >= 16 ? items >= (int64_t)num_sms() * 8
-                               : (U == 1 || (U == 8 && VM != VM_F64)) && items >= (int64_t)num_sms() * 32 && a.split_rows * 4 > a.n_rows;
+    // U = 1, and 8 in FP32: the joint kernel's occupancy is below the walk's
+    // own, which counts where many rows go deep, with U = 1 not far (5M rows of
+    // U{1..29}, FP32, depth 16: 285 and 223 against 240 and 209 us).
+    const bool many = items >= (int64_t)num_sms() * 32, wide = a.split_rows * 4 > a.n_rows;
+    const bool apart = U >= 16 ? many || (VM == VM_F64 && items >= (int64_t)num_sms() * 8)
+                       : U == 8 ? many && wide && VM != VM_F64 : U == 1 && many && wide && mostly_shallow;
     if (items > 0 && apart) {
         const unsigned db = (unsigned)std::min<int64_t>(items, (int64_t)num_sms() * 16);
         jds_deep_kernel<VM><<<db, 256, 0, s>>>(a, items);
@@ -942,11 +943,12 @@ static gbsp_status launch_family(const Mat &A, JdsArgs a, cudaStream_t s) {
         a.split_rows = A.split_rows;
     }
     const int64_t items = A.split_k > 0 ? A.split_items_total : 0;
-    if (u <= 1) launch_row<VM, 1>(a, R, s, items);
-    else if (u <= 2) launch_row<VM, 2>(a, R, s, items);
-    else if (u <= 4) launch_row<VM, 4>(a, R, s, items);
-    else if (u <= 8) launch_row<VM, 8>(a, std::min(R, 2), s, items);
-    else launch_row<VM, 16>(a, 1, s, items);
+    const bool shallow = A.split_k > 0 && 3 * (A.nnz - A.h_jd_ptr[(size_t)A.split_depth]) < A.nnz;
+    if (u <= 1) launch_row<VM, 1>(a, R, s, items, shallow);
+    else if (u <= 2) launch_row<VM, 2>(a, R, s, items, shallow);
+    else if (u <= 4) launch_row<VM, 4>(a, R, s, items, shallow);
+    else if (u <= 8) launch_row<VM, 8>(a, std::min(R, 2), s, items, shallow);
+    else launch_row<VM, 16>(a, 1, s, items, shallow);
     if (A.split_k > 0) {
         const int64_t work = std::max<int64_t>(A.split_wide_rows * 32, A.split_rows - A.split_wide_rows);
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(work, 256), (int64_t)num_sms() * 8));

@@ -53,7 +53,7 @@ def test_split_walk_chunks(perm, dtype):
 def test_split_apart(unroll, dtype):
     """Deep items enough to fill the GPU, on rows most of which go deep: the
     deep items are launched before the walk.  Integer data, any order exact."""
-    n = 60_000
+    n = 400_000 if unroll == 1 else 60_000
     lens = S.randint(3, 1, np.arange(n), 0, 50).astype(np.int64)
     row_ptr = np.zeros(n + 1, np.int64)
     np.cumsum(lens, out=row_ptr[1:])
@@ -63,7 +63,7 @@ def test_split_apart(unroll, dtype):
     x, y0 = S.int_vector(n, 5, 16), S.int_vector(n, 6, 100)
     ref = O.crs_spmv(A, x)
     J = crs(A, dtype).to_jds("NUJDS", "symmetric", unroll=unroll)
-    for depth, chunk in ((1, 1), (9, 1), (49, 8)):
+    for depth, chunk in ((1, 1), (9, 1), (30, 1), (49, 8)):  # (30, 1): few entries deep
         J.split(depth, chunk)
         for limit in (0, 3):
             J.set_grid_limit(limit)
