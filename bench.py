@@ -225,7 +225,7 @@ def kernel_source_hash(kname: str = "SELL") -> str:
 # workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum,
 # a one-pass metric set), keyed by (config, kernel, source hash); a different
 # hash means the kernel changed since and traffic is reported null.
-NCU_TRAFFIC = {(1, "SELL symmetric w=128 u=4", "5597793e0a61"): 1087559936 + 42126336}
+NCU_TRAFFIC = {(1, "SELL symmetric w=128 u=4", "fb14ca38e0d1"): 1087956992 + 41890304}
 
 
 # --------------------------------------------------------------- ours ------

@@ -55,7 +55,7 @@ struct Mat {
     int32_t window = 0;             // SELL: rows per sorting window
 
     // JDS / NUJDS deep-diagonal split (caller workspace): diagonals >= split_depth
-    // are summed in chunks by a separate kernel into ragged partial sums
+    // are summed in chunks by blocks of their own into ragged partial sums
     int32_t split_depth = 0, split_chunk = 0, split_k = 0;
     int64_t split_items_total = 0;
     const int4 *split_table = nullptr;  // per chunk {d_begin, d_end, rows, partial offset}

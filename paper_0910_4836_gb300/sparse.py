@@ -393,7 +393,7 @@ class JDSMatrix(_Product):
         L.check(L.load().gbsp_jds_values(self._h, _vp(crs_val), _stream(stream)), "gbsp_jds_values")
 
     def split(self, depth: int = 64, chunk: int = 128, stream=None) -> None:
-        """Sum diagonals >= depth in chunks by a separate kernel (long rows
+        """Sum diagonals >= depth in chunks by blocks of their own (long rows
         spread over many threads); depth=0 removes the split."""
         lib = L.load()
         if depth == 0:
