@@ -743,11 +743,13 @@ int crs_row_cut(const Mat &A) {
 // and 33, FP32 50, 28 and 25), two for light tails in FP64 (crs_short_kernel),
 // one from five entries on, where heavy tails are as likely, and in FP32, which
 // pays more for the step out of line (rows of mean 2.5 with a log-normal
-// tail: 43 us with one set, 55 with two).
+// tail: 43 us with one set, 55 with two).  One, too, where the rows would not
+// fill the GPU with several (5-point Laplacian, 10,000, 40,000 and 160,000 rows,
+// one / two sets: 2.35 / 2.87, 2.78 / 3.24, 4.40 / 4.16 us).
 int crs_default_rows(const Mat &A) {
     const double mean = row_mean(A);
     if (A.kopt.lanes > 1) return 4;
-    if (mean == 0) return 1;
+    if (mean == 0 || A.n_rows < 100000) return 1;
     if (A.dtype == GBSP_F64) return mean < 1.5 ? 4 : mean < 5 ? 2 : 1;
     return mean < 2.25 ? 4 : 1;
 }

@@ -27,8 +27,12 @@ def test_long_rows(mean, f64, f32):
     assert shape(64, 64 * mean, 1) == (f32, 4)
 
 
-@pytest.mark.parametrize("nnz,f64,f32", [(0, 1, 1), (1, 4, 4), (149, 4, 4), (150, 2, 4), (224, 2, 4), (225, 2, 1),
-                                         (499, 2, 1), (500, 1, 1), (599, 1, 1)])
-def test_short_rows(nnz, f64, f32):
-    assert shape(100, nnz, 0) == (1, f64)
-    assert shape(100, nnz, 1) == (1, f32)
+@pytest.mark.parametrize("hundredths,f64,f32", [(0, 1, 1), (1, 4, 4), (149, 4, 4), (150, 2, 4), (224, 2, 4),
+                                                (225, 2, 1), (499, 2, 1), (500, 1, 1), (599, 1, 1)])
+def test_short_rows(hundredths, f64, f32):
+    """Sets of rows a warp with one lane a row, by the mean in hundredths; one
+    where there are too few rows for several."""
+    for n in (100_000, 99_900):
+        nnz = n // 100 * hundredths
+        assert shape(n, nnz, 0) == (1, f64 if n == 100_000 else 1)
+        assert shape(n, nnz, 1) == (1, f32 if n == 100_000 else 1)
